@@ -1,6 +1,7 @@
 // Host-side objects of libpwave: context, model, stream header, plans.
 #pragma once
 
+#include <list>
 #include <map>
 #include <memory>
 #include <mutex>
@@ -64,6 +65,7 @@ struct Model {
   uint64_t uid = 0;          // unique per loaded model (keys cached workspaces)
   std::vector<float *> allocs;
   std::map<std::string, std::vector<float>> host;
+  std::list<std::vector<float>> lift_host;   // the lifting nets' LiftNetDev::wt_host
   LiftNetDev lift[2][2];   // [row, col][P, U]
   LiftNetDev tlift[2];     // [P, U]
   // post-processing CNN after the inverse transform (present when the blob

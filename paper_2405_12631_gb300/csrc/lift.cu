@@ -6,8 +6,7 @@
 // of the forward transform backwards, so it reconstructs perfectly for any
 // network weights. The CNN residual is conv3x3(1->16), tanh,
 // conv3x3(16->16), tanh, conv3x3(16->1) with zero padding, fused in one
-// kernel per 16x16 output tile (halo of 3, all activations in shared
-// memory). Linear parts: LeGall 5/3 (P = (s[n] + s[n+1]) / 2,
+// kernel per output tile (halo of 3, all activations in shared memory). Linear parts: LeGall 5/3 (P = (s[n] + s[n+1]) / 2,
 // U = (s[n-1] + s[n]) / 4, edges clamped = whole-sample symmetric) for the
 // spatial transform; Haar (P = s, U = s / 2) for the temporal one. Integer
 // mode (lossless) rounds P with floor(v) and U with floor(v + 1/2), which
@@ -24,6 +23,7 @@
 // keep fused multiply-adds and the CUDA tanh.
 #include <cuda_bf16.h>
 
+#include <cstring>
 #include <mutex>
 
 #include "pw_internal.cuh"
@@ -34,49 +34,21 @@
 
 namespace pw {
 
-constexpr int LT = 16;            // output tile
 constexpr int LF = 16;            // CNN channels
+// the tensor-core step's tile
+constexpr int LT = 16;            // output tile
 constexpr int L1 = LT + 4;        // layer-1 region (20)
 constexpr int L2 = LT + 2;        // layer-2 region (18)
 constexpr int LI = LT + 6;        // input region (22)
 
-// Shared memory of one tile. Weights are stored tap-major with the output
-// (or input) channel innermost so that 16 of them come in four broadcast
-// 128-bit loads: w1t[tap][c], w2t[tap][ci][c], w3t[tap][ci].
-struct LiftSmem {
-  alignas(16) float in[LI * LI];
-  alignas(16) float a1[L1 * L1 * LF];
-  alignas(16) float a2[L2 * L2 * LF];
-  alignas(16) float w1t[9 * LF];
-  alignas(16) float w2t[9 * LF * LF];
-  alignas(16) float w3t[9 * LF];
-  alignas(16) float b1[LF];
-  alignas(16) float b2[LF];
-  alignas(16) float b3[4];
-};
-
-__device__ __forceinline__ void ld16(const float *p, float *v) {
-  const float4 *q = reinterpret_cast<const float4 *>(p);
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const float4 f = q[i];
-    v[4 * i] = f.x; v[4 * i + 1] = f.y; v[4 * i + 2] = f.z; v[4 * i + 3] = f.w;
-  }
-}
-
-// acc + w * x: one fused multiply-add, or (kExact) a rounded product and a
-// rounded sum; the activation: CUDA's tanhf, or (kExact) tanh32_spec.
-template <bool kExact>
-__device__ __forceinline__ float mac(float acc, float w, float x) {
-  return kExact ? __fadd_rn(acc, __fmul_rn(w, x)) : fmaf(w, x, acc);
-}
+// The activation: CUDA's tanhf, or (kExact) tanh32_spec.
 template <bool kExact>
 __device__ __forceinline__ float act(float v) {
   return kExact ? tanh32_spec(v) : tanhf(v);
 }
 
-// Two accumulators of mac<kExact> at once (per element the same operations:
-// a fused multiply-add, or (kExact) a rounded product and a rounded sum).
+// Two accumulators at once, acc + w x: per element a fused multiply-add, or
+// (kExact) a rounded product and a rounded sum.
 template <bool kExact>
 __device__ __forceinline__ uint64_t mac2(uint64_t acc, uint64_t w, uint64_t x) {
   return kExact ? add2(acc, mul2(w, x)) : fma2(w, x, acc);
@@ -89,43 +61,19 @@ __device__ __forceinline__ void acc_set(const PlaneAcc &a, int p, int y, int x, 
   a.p[(int64_t)p * a.ps + (int64_t)y * a.rs + (int64_t)x * a.cs] = v;
 }
 
-// Layer 3 of the CNN (conv3x3 16 -> 1 over the 18 x 18 layer-2 region a2,
-// null when the step has no CNN), the linear part and the output of one
-// 16 x 16 tile; thread t handles output (t / 16, t % 16). in: the 22 x 22
-// input region (origin y0 - 3, x0 - 3).
-// rout (optional): the CNN residual of the tile's outputs, already computed.
+// The linear part and the output at (y, x) of a plane: c points at the source
+// sample in the staged input, whose rows are `stride` apart; r_out is the CNN
+// residual.
 template <bool kExact>
-__device__ __forceinline__ void lift_finish(const LiftStepParams &a, int p, int H, int W, int y0,
-                                            int x0, const float *in, const float *a2,
-                                            const float *w3t, const float *b3,
-                                            const float *rout = nullptr) {
-  const int t = threadIdx.x;
-  const int ly = t / LT, lx = t % LT;
-  float r_out = 0.f;
-  if (rout) {
-    r_out = rout[t];
-  } else if (a2) {
-    float v = b3[0];
-    for (int tap = 0; tap < 9; ++tap) {
-      float xv[LF], w[LF];
-      ld16(a2 + ((ly + tap / 3) * L2 + lx + tap % 3) * LF, xv);
-      ld16(w3t + tap * LF, w);
-#pragma unroll
-      for (int ci = 0; ci < LF; ++ci) v = mac<kExact>(v, w[ci], xv[ci]);
-    }
-    r_out = v;
-  }
-  const int y = y0 + ly, x = x0 + lx;
-  if (y >= H || x >= W) return;
-  const float s0 = in[(ly + 3) * LI + lx + 3];
+__device__ __forceinline__ void lift_out(const LiftStepParams &a, int p, int H, int W, int y,
+                                         int x, const float *c, int stride, float r_out) {
+  const float s0 = c[0];
   float lin;
   if (a.lin == LIN_P53) {
-    const float s1 = a.dir == 0 ? (x + 1 < W ? in[(ly + 3) * LI + lx + 4] : s0)
-                                : (y + 1 < H ? in[(ly + 4) * LI + lx + 3] : s0);
+    const float s1 = a.dir == 0 ? (x + 1 < W ? c[1] : s0) : (y + 1 < H ? c[stride] : s0);
     lin = 0.5f * (s0 + s1);
   } else if (a.lin == LIN_U53) {
-    const float sm = a.dir == 0 ? (x > 0 ? in[(ly + 3) * LI + lx + 2] : s0)
-                                : (y > 0 ? in[(ly + 2) * LI + lx + 3] : s0);
+    const float sm = a.dir == 0 ? (x > 0 ? c[-1] : s0) : (y > 0 ? c[-stride] : s0);
     lin = 0.25f * (sm + s0);
   } else if (a.lin == LIN_ID) {
     lin = s0;
@@ -142,117 +90,208 @@ __device__ __forceinline__ void lift_finish(const LiftStepParams &a, int p, int 
   if (a.copy.p) acc_set(a.copy, p, y, x, s0);
 }
 
-template <bool kExact>
-__global__ void __launch_bounds__(256) k_lift_step(LiftStepParams a) {
-  extern __shared__ float smem_raw[];
-  LiftSmem &S = *reinterpret_cast<LiftSmem *>(smem_raw);
+// One lifting step on FP32 cores, one TW x TH output tile per block.
+//
+// What bounds it: the FP32 pipe. Layer 2 is 2304 of the 2592 multiply-adds
+// of a sample (in the exact mode each is a product and a sum, and the 32
+// tanh32_spec of a sample cost a third as much again). So the tile is chosen
+// for layer 2: its region, one wider than the tile on every side, is 512
+// positions for 30 x 14 (a 22 % surplus, two positions x 16 channels per
+// thread, every lane busy) and 128 for 14 x 6 (one position x 8 channels),
+// the small tile for planes that do not fill the chip with large ones.
+// Activations lie in four planes of 4 channels (16 bytes per position):
+// neighbouring lanes read neighbouring 16 bytes, where a 64-byte pixel cost
+// four times the shared-memory passes. Layer 2's result overwrites layer
+// 1's slab once every thread holds its own, so four blocks share an SM.
+// Layer 2's weights are the same for every lane: the large tile reads them
+// from the kernel's parameters (constant bank), since broadcast loads from
+// shared memory return 16 bytes to each of 32 lanes and had the port busy
+// for longer than the arithmetic; the small tile, whose threads split the
+// channels, reads shared memory (11 us against 16 us a launch).
+// Measured: 2 lossless 3840x2160 12-bit RGB images, all steps, 51.7 ms (16 x
+// 16 tile, 64-byte pixels, 162 of 256 threads in layer 2, tanh by branches)
+// -> 28.2 -> 23.6 ms with the weights as parameters; forward lifting of 12
+// 768x512 RGB images 10.7 -> 6.7 -> 5.1 ms; a 250x333 plane, 24 steps, 0.67
+// -> 0.27 ms (small tile).
+// Every layer's per-element operation order is the definition's: bias, then
+// tap by tap, input channel by input channel (channels or outputs in packed
+// FP32 pairs, each element rounded as its scalar operation).
+template <int TW, int TH>
+struct LiftCfg {
+  static constexpr int IW = TW + 6, IH = TH + 6;              // input region
+  static constexpr int W1 = TW + 4, H1 = TH + 4, N1 = W1 * H1;   // layer-1 region
+  static constexpr int W2 = TW + 2, H2 = TH + 2, N2 = W2 * H2;   // layer-2 region
+  static constexpr int NO = TW * TH;
+  static constexpr int PP = N2 >= 512 ? N2 / 256 : 1;         // layer-2 positions per thread
+  static constexpr int CH = 16 * N2 / (256 * PP);             // and channels
+  static_assert(PP * CH * 256 == 16 * N2 && (CH == 16 || CH == 8), "layer-2 work split");
+  static_assert(NO <= 512, "outputs per thread");
+  struct Smem {
+    alignas(16) float act[4 * N1 * 4];   // [channel / 4][position][channel % 4]
+    alignas(16) float wt[kLiftSmall + (CH == 16 ? 0 : kLiftW2)];
+    alignas(16) float in[IW * IH];
+  };
+  // layer 2's weights as a kernel parameter (unused by the small tile)
+  struct Wt2 {
+    alignas(16) float v[CH == 16 ? kLiftW2 : 4];
+  };
+};
+
+template <bool kExact, int TW, int TH>
+__global__ void __launch_bounds__(256, 4) k_lift_step(
+    const __grid_constant__ LiftStepParams a,
+    const __grid_constant__ typename LiftCfg<TW, TH>::Wt2 w2p) {
+  using C = LiftCfg<TW, TH>;
+  extern __shared__ __align__(16) uint8_t lift_smem[];
+  typename C::Smem &S = *reinterpret_cast<typename C::Smem *>(lift_smem);
+  float4 *act4 = reinterpret_cast<float4 *>(S.act);
+  const float *w1t = S.wt, *w3t = S.wt + 144, *b1 = S.wt + 288, *b2 = S.wt + 304;
   const int t = threadIdx.x;
   const int p = blockIdx.z;
-  const int tiles_x = (a.W + LT - 1) / LT;
-  const int y0 = (blockIdx.x / tiles_x) * LT, x0 = (blockIdx.x % tiles_x) * LT;
+  const int tiles_x = (a.W + TW - 1) / TW;
+  const int y0 = (blockIdx.x / tiles_x) * TH, x0 = (blockIdx.x % tiles_x) * TW;
   const bool cnn = a.net.w1 != nullptr;
   int H, W;
   lift_extent(a, p, H, W);
   if (y0 >= H || x0 >= W) return;  // a tile beyond this plane of a ragged batch
 
-  for (int e = t; e < LI * LI; e += 256) {
-    int yy = y0 + e / LI - 3, xx = x0 + e % LI - 3;
+  for (int e = t; e < C::IW * C::IH; e += 256) {
+    const int yy = y0 + e / C::IW - 3, xx = x0 + e % C::IW - 3;
     S.in[e] = (yy >= 0 && yy < H && xx >= 0 && xx < W) ? acc_get(a.src, p, yy, xx) : 0.f;
   }
-  if (cnn) {
-    for (int e = t; e < LF * 9; e += 256) {
-      const int c = e / 9, tap = e % 9;  // source [c][tap]
-      S.w1t[tap * LF + c] = a.net.w1[e];
-      S.w3t[tap * LF + c] = a.net.w3[e];
-    }
-    for (int e = t; e < LF * LF * 9; e += 256) {
-      const int c = e / (LF * 9), ci = (e / 9) % LF, tap = e % 9;  // source [c][ci][tap]
-      S.w2t[(tap * LF + ci) * LF + c] = a.net.w2[e];
-    }
-    if (t < LF) { S.b1[t] = a.net.b1[t]; S.b2[t] = a.net.b2[t]; }
-    if (t == 0) S.b3[0] = a.net.b3[0];
-  }
+  if (cnn)
+    for (int e = t; e < (int)(sizeof(S.wt) / 16); e += 256)
+      reinterpret_cast<float4 *>(S.wt)[e] = __ldg(reinterpret_cast<const float4 *>(a.net.wt) + e);
   __syncthreads();
+  float res[2] = {0.f, 0.f};   // CNN residual of outputs t and t + 256
   if (cnn) {
-    // layer 1 on the 20 x 20 region (origin y0 - 2, x0 - 2)
-    for (int e = t; e < L1 * L1; e += 256) {
-      const int ly = e / L1, lx = e % L1;
+    // layer 1: one position and 8 channels per item
+    for (int it = t; it < 2 * C::N1; it += 256) {
+      const int g = it >= C::N1 ? 1 : 0, pos = it - g * C::N1;
+      const int ly = pos / C::W1, lx = pos % C::W1;
       const int yy = y0 + ly - 2, xx = x0 + lx - 2;
       const bool inside = yy >= 0 && yy < H && xx >= 0 && xx < W;
-      // output channels in pairs (packed FP32): each accumulator sees the
-      // same sequence of operations as one mac<kExact> chain
-      uint64_t accp[LF / 2];
+      uint64_t accp[4];
 #pragma unroll
-      for (int c = 0; c < LF / 2; ++c) accp[c] = f2pack(S.b1[2 * c], S.b1[2 * c + 1]);
+      for (int k = 0; k < 4; ++k) accp[k] = f2pack(b1[8 * g + 2 * k], b1[8 * g + 2 * k + 1]);
 #pragma unroll
       for (int tap = 0; tap < 9; ++tap) {
-        const float iv = S.in[(ly + tap / 3) * LI + lx + tap % 3];
+        const float iv = S.in[(ly + tap / 3) * C::IW + lx + tap % 3];
         const uint64_t xv = f2pack(iv, iv);
-        const uint64_t *wp = reinterpret_cast<const uint64_t *>(S.w1t + tap * LF);
-#pragma unroll
-        for (int c = 0; c < LF / 2; ++c) accp[c] = mac2<kExact>(accp[c], wp[c], xv);
+        const ulonglong2 *wp = reinterpret_cast<const ulonglong2 *>(w1t + tap * LF + 8 * g);
+        const ulonglong2 wa = wp[0], wb = wp[1];
+        accp[0] = mac2<kExact>(accp[0], wa.x, xv);
+        accp[1] = mac2<kExact>(accp[1], wa.y, xv);
+        accp[2] = mac2<kExact>(accp[2], wb.x, xv);
+        accp[3] = mac2<kExact>(accp[3], wb.y, xv);
       }
-      float acc[LF];
 #pragma unroll
-      for (int c = 0; c < LF / 2; ++c) f2unpack(accp[c], acc[2 * c], acc[2 * c + 1]);
-      float4 *dst = reinterpret_cast<float4 *>(S.a1 + e * LF);
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        dst[i] = inside ? make_float4(act<kExact>(acc[4 * i]), act<kExact>(acc[4 * i + 1]),
-                                      act<kExact>(acc[4 * i + 2]), act<kExact>(acc[4 * i + 3]))
-                        : make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int k = 0; k < 2; ++k) {
+        float v[4];
+        f2unpack(accp[2 * k], v[0], v[1]);
+        f2unpack(accp[2 * k + 1], v[2], v[3]);
+        act4[(2 * g + k) * C::N1 + pos] =
+            inside ? make_float4(act<kExact>(v[0]), act<kExact>(v[1]), act<kExact>(v[2]),
+                                 act<kExact>(v[3]))
+                   : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
     }
     __syncthreads();
-    // layer 2 on the 18 x 18 region (origin y0 - 1, x0 - 1): 324 positions,
-    // two per thread (threads 0..161) so that every weight load feeds 32 FMAs
-    constexpr int kHalf = L2 * L2 / 2;
-    if (t < kHalf) {
-      const int e0 = t, e1 = t + kHalf;
-      const int ly0 = e0 / L2, lx0 = e0 % L2, ly1 = e1 / L2, lx1 = e1 % L2;
-      // output channels in pairs (packed FP32), as in layer 1
-      uint64_t p0[LF / 2], p1[LF / 2];
+    // layer 2: positions q + 256 i, channels c0 .. c0 + CH - 1
+    {
+      const int c0 = C::CH == 8 && t >= 128 ? 8 : 0;
+      const int q = C::CH == 8 ? (t & 127) : t;
+      uint64_t acc[C::PP][C::CH / 2];
+      int base[C::PP];
 #pragma unroll
-      for (int c = 0; c < LF / 2; ++c) p0[c] = p1[c] = f2pack(S.b2[2 * c], S.b2[2 * c + 1]);
+      for (int i = 0; i < C::PP; ++i) {
+        const int e = q + 256 * i;
+        base[i] = (e / C::W2) * C::W1 + e % C::W2;
+#pragma unroll
+        for (int k = 0; k < C::CH / 2; ++k)
+          acc[i][k] = f2pack(b2[c0 + 2 * k], b2[c0 + 2 * k + 1]);
+      }
+#pragma unroll 1
       for (int tap = 0; tap < 9; ++tap) {
-        float in0v[LF], in1v[LF];
-        ld16(S.a1 + ((ly0 + tap / 3) * L1 + lx0 + tap % 3) * LF, in0v);
-        ld16(S.a1 + ((ly1 + tap / 3) * L1 + lx1 + tap % 3) * LF, in1v);
+        const int off = (tap / 3) * C::W1 + tap % 3;
+        const float *wrow = C::CH == 16 ? w2p.v + tap * LF * LF
+                                        : S.wt + kLiftSmall + tap * LF * LF + c0;
 #pragma unroll
-        for (int ci = 0; ci < LF; ++ci) {
-          const uint64_t *wp = reinterpret_cast<const uint64_t *>(S.w2t + (tap * LF + ci) * LF);
-          const uint64_t x0 = f2pack(in0v[ci], in0v[ci]), x1 = f2pack(in1v[ci], in1v[ci]);
+        for (int g = 0; g < 4; ++g) {
+          float xv[C::PP][4];
 #pragma unroll
-          for (int c = 0; c < LF / 2; ++c) {
-            const uint64_t w = wp[c];
-            p0[c] = mac2<kExact>(p0[c], w, x0);
-            p1[c] = mac2<kExact>(p1[c], w, x1);
+          for (int i = 0; i < C::PP; ++i) {
+            const float4 f = act4[g * C::N1 + base[i] + off];
+            xv[i][0] = f.x; xv[i][1] = f.y; xv[i][2] = f.z; xv[i][3] = f.w;
+          }
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const ulonglong2 *wp =
+                reinterpret_cast<const ulonglong2 *>(wrow + (4 * g + e) * LF);
+#pragma unroll
+            for (int k = 0; k < C::CH / 4; ++k) {
+              const ulonglong2 w = wp[k];
+#pragma unroll
+              for (int i = 0; i < C::PP; ++i) {
+                const uint64_t xx = f2pack(xv[i][e], xv[i][e]);
+                acc[i][2 * k] = mac2<kExact>(acc[i][2 * k], w.x, xx);
+                acc[i][2 * k + 1] = mac2<kExact>(acc[i][2 * k + 1], w.y, xx);
+              }
+            }
           }
         }
       }
-      float acc0[LF], acc1[LF];
+      __syncthreads();   // layer 1's slab is consumed: layer 2's goes over it
 #pragma unroll
-      for (int c = 0; c < LF / 2; ++c) {
-        f2unpack(p0[c], acc0[2 * c], acc0[2 * c + 1]);
-        f2unpack(p1[c], acc1[2 * c], acc1[2 * c + 1]);
-      }
-      const int yy0 = y0 + ly0 - 1, xx0 = x0 + lx0 - 1, yy1 = y0 + ly1 - 1, xx1 = x0 + lx1 - 1;
-      const bool in0 = yy0 >= 0 && yy0 < H && xx0 >= 0 && xx0 < W;
-      const bool in1 = yy1 >= 0 && yy1 < H && xx1 >= 0 && xx1 < W;
-      float4 *d0 = reinterpret_cast<float4 *>(S.a2 + e0 * LF);
-      float4 *d1 = reinterpret_cast<float4 *>(S.a2 + e1 * LF);
+      for (int i = 0; i < C::PP; ++i) {
+        const int e = q + 256 * i;
+        const int yy = y0 + e / C::W2 - 1, xx = x0 + e % C::W2 - 1;
+        const bool inside = yy >= 0 && yy < H && xx >= 0 && xx < W;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        d0[i] = in0 ? make_float4(act<kExact>(acc0[4 * i]), act<kExact>(acc0[4 * i + 1]),
-                                  act<kExact>(acc0[4 * i + 2]), act<kExact>(acc0[4 * i + 3]))
-                    : make_float4(0.f, 0.f, 0.f, 0.f);
-        d1[i] = in1 ? make_float4(act<kExact>(acc1[4 * i]), act<kExact>(acc1[4 * i + 1]),
-                                  act<kExact>(acc1[4 * i + 2]), act<kExact>(acc1[4 * i + 3]))
-                    : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int k = 0; k < C::CH / 4; ++k) {
+          float v[4];
+          f2unpack(acc[i][2 * k], v[0], v[1]);
+          f2unpack(acc[i][2 * k + 1], v[2], v[3]);
+          act4[(c0 / 4 + k) * C::N2 + e] =
+              inside ? make_float4(act<kExact>(v[0]), act<kExact>(v[1]), act<kExact>(v[2]),
+                                   act<kExact>(v[3]))
+                     : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
       }
     }
     __syncthreads();
+    // layer 3: outputs t and t + 256 as one packed pair
+    {
+      const int oa = min(t, C::NO - 1), ob = min(t + 256, C::NO - 1);
+      const int pa = (oa / TW) * C::W2 + oa % TW, pb = (ob / TW) * C::W2 + ob % TW;
+      const float b3 = S.wt[320];
+      uint64_t v = f2pack(b3, b3);
+#pragma unroll 1
+      for (int tap = 0; tap < 9; ++tap) {
+        const int off = (tap / 3) * C::W2 + tap % 3;
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          const float4 w = *reinterpret_cast<const float4 *>(w3t + tap * LF + 4 * g);
+          const float4 xa = act4[g * C::N2 + pa + off];
+          const float4 xb = C::NO > 256 ? act4[g * C::N2 + pb + off] : xa;
+          v = mac2<kExact>(v, f2pack(w.x, w.x), f2pack(xa.x, xb.x));
+          v = mac2<kExact>(v, f2pack(w.y, w.y), f2pack(xa.y, xb.y));
+          v = mac2<kExact>(v, f2pack(w.z, w.z), f2pack(xa.z, xb.z));
+          v = mac2<kExact>(v, f2pack(w.w, w.w), f2pack(xa.w, xb.w));
+        }
+      }
+      f2unpack(v, res[0], res[1]);
+    }
   }
-  lift_finish<kExact>(a, p, H, W, y0, x0, S.in, cnn ? S.a2 : nullptr, S.w3t, S.b3);
+#pragma unroll
+  for (int i = 0; i < (C::NO > 256 ? 2 : 1); ++i) {
+    const int o = t + 256 * i;
+    if (o >= C::NO) break;
+    const int ly = o / TW, lx = o % TW;
+    const int y = y0 + ly, x = x0 + lx;
+    if (y < H && x < W)
+      lift_out<kExact>(a, p, H, W, y, x, S.in + (ly + 3) * C::IW + lx + 3, C::IW, res[i]);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -483,7 +522,9 @@ __global__ void __launch_bounds__(256, 6) k_lift_tc(LiftStepParams a) {
     __syncwarp();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tbase), "r"(kCols));
   }
-  if (ok) lift_finish<false>(a, p, H, W, y0, x0, S.in, nullptr, nullptr, nullptr, S.rout);
+  const int oy = y0 + t / LT, ox = x0 + t % LT;
+  if (ok && oy < H && ox < W)
+    lift_out<false>(a, p, H, W, oy, ox, S.in + (t / LT + 3) * LI + t % LT + 3, LI, S.rout[t]);
 }
 
 // Component planes [B][nc][Hp][Wp] -> interleaved samples (crop, inverse
@@ -582,6 +623,21 @@ static int grid_for(int64_t n) {
   return (int)(g > 152 * 32 ? 152 * 32 : (g < 1 ? 1 : g));
 }
 
+template <bool kExact, int TW, int TH>
+static void launch_lift_tile(const LiftStepParams &a, cudaStream_t st) {
+  constexpr int smem = (int)sizeof(typename LiftCfg<TW, TH>::Smem);
+  static std::atomic<uint64_t> attr{0};
+  once_per_device(attr, [] {
+    cudaFuncSetAttribute(k_lift_step<kExact, TW, TH>,
+                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  });
+  dim3 grid(((a.H + TH - 1) / TH) * ((a.W + TW - 1) / TW), 1, a.P);
+  typename LiftCfg<TW, TH>::Wt2 w2;
+  if (LiftCfg<TW, TH>::CH == 16 && a.net.wt_host)
+    std::memcpy(w2.v, a.net.wt_host + kLiftSmall, sizeof(w2.v));
+  k_lift_step<kExact, TW, TH><<<grid, 256, smem, st>>>(a, w2);
+}
+
 void launch_lift_step(const LiftStepParams &a, cudaStream_t st) {
   if (a.tc && a.net.w1 && a.round == 0) {
     static std::atomic<uint64_t> attr_tc{0};
@@ -594,18 +650,17 @@ void launch_lift_step(const LiftStepParams &a, cudaStream_t st) {
     k_lift_tc<<<grid, 256, sizeof(LiftTcSmem) + 1024, st>>>(a);
     return;
   }
-  static std::atomic<uint64_t> attr{0};
-  once_per_device(attr, [] {
-    cudaFuncSetAttribute(k_lift_step<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)sizeof(LiftSmem));
-    cudaFuncSetAttribute(k_lift_step<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)sizeof(LiftSmem));
-  });
-  const int tiles = ((a.H + LT - 1) / LT) * ((a.W + LT - 1) / LT);
-  dim3 grid(tiles, 1, a.P);
+  // large tiles where they fill the chip, small ones (a quarter of the work
+  // per thread, half as much surplus again) where latency counts
+  const int64_t big = (int64_t)((a.H + 13) / 14) * ((a.W + 29) / 30) * a.P;
   // integer (lossless) steps take the exact operation sequence
-  if (a.round != 0) k_lift_step<true><<<grid, 256, sizeof(LiftSmem), st>>>(a);
-  else k_lift_step<false><<<grid, 256, sizeof(LiftSmem), st>>>(a);
+  if (big > sm_count()) {
+    if (a.round != 0) launch_lift_tile<true, 30, 14>(a, st);
+    else launch_lift_tile<false, 30, 14>(a, st);
+  } else {
+    if (a.round != 0) launch_lift_tile<true, 14, 6>(a, st);
+    else launch_lift_tile<false, 14, 6>(a, st);
+  }
 }
 void launch_colour_out(const float *planes, int B, int nc, int Hp, int Wp, int H, int W,
                        int colour, int bitdepth, void *out, int64_t img_stride,

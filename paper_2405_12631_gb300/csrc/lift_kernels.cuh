@@ -18,7 +18,12 @@ struct LiftNetDev {
   // BF16 MMA B operands of layers 2 and 3 for the tensor-core step, packed
   // [tap][2 channel groups][16 outputs][8] (layer 3: output 0, rest zero)
   const void *w2b, *w3b;
+  // the FP32 step's weights, on the device and on the host (the model's):
+  // w1 [tap][c], w3 [tap][ci], b1, b2, b3 and padding (kLiftSmall floats),
+  // then w2 [tap][ci][c]
+  const float *wt, *wt_host;
 };
+constexpr int kLiftSmall = 144 + 144 + 16 + 16 + 4, kLiftW2 = 9 * 16 * 16;
 
 enum { LIN_P53 = 0, LIN_U53 = 1, LIN_ID = 2, LIN_HALF = 3, LIN_ZERO = 4 };
 

@@ -180,6 +180,22 @@ int Model::load(pw_ctx *c, const void *blob, size_t n) {
         !get(p + "w2", {16, 16, 3, 3}, w2) || !get(p + "b2", {16}, b2) ||
         !get(p + "w3", {1, 16, 3, 3}, w3) || !get(p + "b3", {1}, b3))
       return false;
+    {
+      lift_host.emplace_back(kLiftSmall + kLiftW2, 0.f);
+      std::vector<float> &wt = lift_host.back();
+      for (int c = 0; c < 16; ++c)
+        for (int tap = 0; tap < 9; ++tap) {
+          wt[tap * 16 + c] = w1[c * 9 + tap];
+          for (int ci = 0; ci < 16; ++ci)
+            wt[kLiftSmall + (tap * 16 + ci) * 16 + c] = w2[(c * 16 + ci) * 9 + tap];
+          wt[144 + tap * 16 + c] = w3[c * 9 + tap];
+        }
+      std::copy(b1.begin(), b1.end(), wt.begin() + 288);
+      std::copy(b2.begin(), b2.end(), wt.begin() + 304);
+      wt[320] = b3[0];
+      n.wt = up(wt);
+      n.wt_host = wt.data();
+    }
     n.w1 = up(w1); n.b1 = up(b1); n.w2 = up(w2); n.b2 = up(b2); n.w3 = up(w3); n.b3 = up(b3);
     {
       // packed BF16 B operands: [tap][ci / 8][c][ci % 8]
