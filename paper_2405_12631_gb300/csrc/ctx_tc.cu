@@ -14,9 +14,9 @@
 // processed in K-blocks of 64 (32) channels. Weights of the CTA's N block
 // stay resident in shared memory for the whole persistent kernel.
 // Warp roles: warp 0 = TMA producer, warp 1 = MMA issuer (and TMEM owner),
-// warps 2-5 = epilogue (one TMEM lane quadrant each). Accumulators are
-// double-buffered in TMEM so the epilogue of one tile overlaps the MMAs of
-// the next. Every wait is bounded: on expiry the kernel sets an error flag,
+// the others = epilogue (8 or 16 warps, by TMEM lane quadrant and part of the
+// columns). Four accumulators in TMEM let the epilogue of a tile overlap the
+// MMAs of the next ones. Every wait is bounded: on expiry the kernel sets an error flag,
 // lets in-flight copies land, frees its tensor memory and returns.
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -29,6 +29,7 @@
 #include <cmath>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 
 #include "ctx_tc.h"
 #include "prof.h"
@@ -115,7 +116,6 @@ struct TcConvArgs {
   int ncta, nb;
   int tiles_x, tiles_y, tiles;  // tiles per N block
   int step_dx, step_dy, step_dp;  // the CTA stride in (tiles_x, tiles_y) digits
-  int pairs;                      // MMA issue of two tiles per round (see the issuer)
   int stages, halo_x, halo_y;
   uint32_t stage_bytes, w_bytes;
   const __nv_bfloat16 *wt;      // [nb][kblock][tap][kb/8][ncta][8]
@@ -136,8 +136,10 @@ struct TcConvArgs {
   int out_G, out_goff;
   const __nv_bfloat16 *res;
   int res_G, res_goff;
-  // ConvLSTM cell state, BF16 [P][H][W][C] (previous subband's resolution
-  // for c_prev)
+  // ConvLSTM cell state, BF16 [P][C / 8][H][W][8] (previous subband's
+  // resolution for c_prev); a warp's 16-byte accesses are then runs of 128
+  // bytes (pixel-major ones touched 32 lines each: FP8 gates 5.67 -> 5.08 ms
+  // per batch of 24)
   const __nv_bfloat16 *c_prev;
   __nv_bfloat16 *c_new;
   int up, first, C;
@@ -219,6 +221,19 @@ __device__ __forceinline__ void load_bf16x8(const __nv_bfloat16 *p, float *v) {
   }
 }
 
+// 8 floats -> 8 E4M3 bytes (round to nearest, saturating), one 8-byte store
+__device__ __forceinline__ void store_fp8x8(uint8_t *p, const float *v) {
+  uint32_t w[2];
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const uint32_t lo = __nv_cvt_float2_to_fp8x2(make_float2(v[4 * i], v[4 * i + 1]),
+                                                 __NV_SATFINITE, __NV_E4M3);
+    const uint32_t hi = __nv_cvt_float2_to_fp8x2(make_float2(v[4 * i + 2], v[4 * i + 3]),
+                                                 __NV_SATFINITE, __NV_E4M3);
+    w[i] = lo | (hi << 16);
+  }
+  *reinterpret_cast<uint2 *>(p) = make_uint2(w[0], w[1]);
+}
 // 16 floats -> 16 E4M3 bytes (round to nearest, saturating), one 16-byte store
 __device__ __forceinline__ void store_fp8x16(uint8_t *p, const float *v) {
   uint32_t w[4];
@@ -233,12 +248,31 @@ __device__ __forceinline__ void store_fp8x16(uint8_t *p, const float *v) {
   *reinterpret_cast<uint4 *>(p) = make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-__device__ __forceinline__ void mma_fp8(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc,
-                                        uint32_t accum) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-      "l"(a), "l"(b), "r"(idesc), "r"(accum));
+// One MMA whose operand descriptors are given as 32-bit halves: the high ones
+// are constants and the address field never carries out of the low ones, so
+// an offset is one 32-bit addition.
+template <bool F8>
+__device__ __forceinline__ void mma_lo(uint32_t d, uint32_t alo, uint32_t ahi, uint32_t blo,
+                                       uint32_t bhi, uint32_t idesc, uint32_t accum) {
+  if constexpr (F8)
+    asm volatile(
+        "{\n .reg .pred p;\n .reg .b64 a, b;\n setp.ne.b32 p, %6, 0;\n"
+        " mov.b64 a, {%1, %2};\n mov.b64 b, {%3, %4};\n"
+        " tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], a, b, %5, p;\n}\n" ::"r"(d),
+        "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(accum));
+  else
+    asm volatile(
+        "{\n .reg .pred p;\n .reg .b64 a, b;\n setp.ne.b32 p, %6, 0;\n"
+        " mov.b64 a, {%1, %2};\n mov.b64 b, {%3, %4};\n"
+        " tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n}\n" ::"r"(d),
+        "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(accum));
+}
+// One lane of a converged warp.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n"
+               : "=r"(r));
+  return r != 0;
 }
 
 // pipeline stages at most (the barrier arrays below hold this many)
@@ -249,13 +283,14 @@ constexpr int kMaxStages = 24;
 // weights and the stages
 constexpr int kConvHeader = 8192;
 
-// Epilogue warps: 16 (four per TMEM lane quadrant, 16 columns each) for the
-// 1x1 plain stores of 64 columns, whose short epilogue is latency-bound
-// (measured: 1x1 class 9.04 -> 8.53 ms per batch of 24; the 3x3 stores lost
-// as much, their MMA and load warps need the issue slots), else 8 (two per
-// quadrant, NCTA / 2 columns each).
+// Epilogue warps: 16 (four per TMEM lane quadrant) for the plain stores of 64
+// columns and the gates of 128, whose epilogues are the longer side and
+// latency-bound (per batch of 24: 1x1 class 9.04 -> 8.53 ms; with the issue
+// loop below, FP8 conv 1 4.38 -> 4.28 ms, FP8 gates 5.08 -> 4.75 ms), else 8
+// (two per quadrant, NCTA / 2 columns each: the BF16 gates' 64 columns hold
+// 16 channels, and their MMAs are the longer side).
 __host__ __device__ constexpr int conv_epi_warps(int ks, int epi, int ncta) {
-  return (ks == 1 && (epi == TE_STORE || epi == TE_STOREV) && ncta == 64) ? 16 : 8;
+  return ((epi == TE_STORE || epi == TE_STOREV) && ncta == 64) || (epi == TE_LSTM && ncta == 128) ? 16 : 8;
 }
 __host__ __device__ constexpr int conv_threads(int ks, int epi, int ncta) {
   return 64 + 32 * conv_epi_warps(ks, epi, ncta);
@@ -300,7 +335,8 @@ __global__ void __launch_bounds__(conv_threads(KS, EPI, NCTA), 1) k_conv_tc(cons
   constexpr bool STORE = EPI == TE_STORE || EPI == TE_STOREV;
   constexpr bool HV = EPI == TE_LSTM || EPI == TE_STOREV;
   constexpr bool VMERGE = EPI == TE_LSTM;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // (the shuffle tells the compiler that the warp index is uniform)
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const int nb = blockIdx.x % a.nb;
   const int cta = blockIdx.x / a.nb;
   const int nctas = gridDim.x / a.nb;
@@ -381,73 +417,56 @@ __global__ void __launch_bounds__(conv_threads(KS, EPI, NCTA), 1) k_conv_tc(cons
     int stage = 0;
     uint32_t phase = 0;
     int issued = 0;
-    // Tiles come in rounds of one, or two (paired issue: the MMA warp
-    // interleaves two tiles into two accumulators) whose stages alternate:
-    // K-step k of the first tile, K-step k of the second, k + 1, ...
-    const bool pairs = a.pairs && a.stages >= 2;
     TileIter ti(cta, a.tiles_x, a.tiles_y);
-    for (int t = cta; t < a.tiles && !*s_abort;) {
-      const bool two = pairs && t + nctas < a.tiles;
-      TileIter t1 = ti;
-      t1.next(a.step_dx, a.step_dy, a.step_dp, a.tiles_x, a.tiles_y);   // tile t + nctas
-      bool stop = false;
-      for (int kbi = 0; kbi < a.nkb && !stop; ++kbi) {
-        for (int u = 0; u < (two ? 2 : 1); ++u) {
-          const TileIter &tt = u ? t1 : ti;
-          const int tx = tt.tx, ty = tt.ty, p = tt.p;
-          if (!mbar_wait(&empty[stage], phase ^ 1, s_abort, 500)) { stop = true; break; }
-          const bool vk = HV && kbi == 0;    // the stage holds the v block
-          const bool vsep = vk && !VMERGE;   // ... and nothing else
-          const uint32_t hb = VMERGE ? a.hstage_bytes : a.stage_bytes;
-          mbar_expect_tx(&full[stage], vsep ? a.vstage_bytes : vk ? hb + a.vstage_bytes : hb);
-          if constexpr (EPI == TE_HEADC) {
-            // compact head: K-step kbi = a.tps taps (9 / a.tps steps per
-            // tile), one box per tap of cR rows x cJ positions x all
-            // channels (one 128-row swizzled K-major slab). Output (row, j)
-            // of the tile is at y = 2 (i0 + row) + par, x = aph + 4 (j0 + j);
-            // tap (dy, dx) reads row 2 (i0 + row) + v, v = par + dy, through
-            // the map of rows of parity v & 1 (index i0 + row + (v >> 1)),
-            // and column 4 (j0 + j) + w, w = aph + dx, as phase w & 3 of
-            // position j0 + j + (w >> 2). Out-of-range boxes read zeros (the
-            // padding).
-            const int par = ty & 1, i0 = (ty >> 1) * a.cR, j0 = tx * a.cJ;
-            const int aph = step_phase(a.step, par);
-            const uint32_t box = a.stage_bytes / a.tps;
-            for (int k = 0; k < a.tps; ++k) {
-              const int tap = kbi * a.tps + k;
-              const int v = par + tap / 3 - 1, w = aph + tap % 3 - 1;
-              const CUtensorMap *mp = (v & 1) ? &tmap1 : &tmap;
-              tma_load_5d(stg + (size_t)stage * a.stage_bytes + k * box, mp, &full[stage], 0,
-                          j0 + (w >> 2), w & 3, i0 + (v >> 1), p);
-            }
-          } else {
-            // K-blocks [0, nkb0) come through tmap (group offset in_goff),
-            // the rest through tmap1 (groups counted from 0); innermost
-            // coordinate = pixel x * 8 channels (a multiple of 8 elements =
-            // 16 bytes, also when negative at the left border)
-            if (vk)
-              tma_load_4d(stg + (size_t)stage * a.stage_bytes + a.hstage_bytes, &tmap,
-                          &full[stage], (tx * kTileW - R) * 8, ty * kTileH - R, 0, p);
-            if (vsep) {
-            } else if (kbi < a.nkb0)
-              tma_load_4d(stg + (size_t)stage * a.stage_bytes, &tmap, &full[stage],
-                          (tx * kTileW - R) * EPG, ty * kTileH - R, a.in_goff + kbi * GPK, p);
-            else
-              tma_load_4d(stg + (size_t)stage * a.stage_bytes, &tmap1, &full[stage],
-                          (tx * kTileW - R) * EPG, ty * kTileH - R,
-                          a.in1_goff + (kbi - a.nkb0) * GPK, p);
+    bool stop = false;
+    for (int t = cta; t < a.tiles && !stop && !*s_abort;
+         t += nctas, ti.next(a.step_dx, a.step_dy, a.step_dp, a.tiles_x, a.tiles_y)) {
+      const int tx = ti.tx, ty = ti.ty, p = ti.p;
+      for (int kbi = 0; kbi < a.nkb; ++kbi) {
+        if (!mbar_wait(&empty[stage], phase ^ 1, s_abort, 500)) { stop = true; break; }
+        const bool vk = HV && kbi == 0;    // the stage holds the v block
+        const bool vsep = vk && !VMERGE;   // ... and nothing else
+        const uint32_t hb = VMERGE ? a.hstage_bytes : a.stage_bytes;
+        mbar_expect_tx(&full[stage], vsep ? a.vstage_bytes : vk ? hb + a.vstage_bytes : hb);
+        if constexpr (EPI == TE_HEADC) {
+          // compact head: K-step kbi = a.tps taps (9 / a.tps steps per
+          // tile), one box per tap of cR rows x cJ positions x all
+          // channels (one 128-row swizzled K-major slab). Output (row, j)
+          // of the tile is at y = 2 (i0 + row) + par, x = aph + 4 (j0 + j);
+          // tap (dy, dx) reads row 2 (i0 + row) + v, v = par + dy, through
+          // the map of rows of parity v & 1 (index i0 + row + (v >> 1)),
+          // and column 4 (j0 + j) + w, w = aph + dx, as phase w & 3 of
+          // position j0 + j + (w >> 2). Out-of-range boxes read zeros (the
+          // padding).
+          const int par = ty & 1, i0 = (ty >> 1) * a.cR, j0 = tx * a.cJ;
+          const int aph = step_phase(a.step, par);
+          const uint32_t box = a.stage_bytes / a.tps;
+          for (int k = 0; k < a.tps; ++k) {
+            const int tap = kbi * a.tps + k;
+            const int v = par + tap / 3 - 1, w = aph + tap % 3 - 1;
+            const CUtensorMap *mp = (v & 1) ? &tmap1 : &tmap;
+            tma_load_5d(stg + (size_t)stage * a.stage_bytes + k * box, mp, &full[stage], 0,
+                        j0 + (w >> 2), w & 3, i0 + (v >> 1), p);
           }
-          ++issued;
-          if (++stage == a.stages) { stage = 0; phase ^= 1; }
+        } else {
+          // K-blocks [0, nkb0) come through tmap (group offset in_goff),
+          // the rest through tmap1 (groups counted from 0); innermost
+          // coordinate = pixel x * 8 channels (a multiple of 8 elements =
+          // 16 bytes, also when negative at the left border)
+          if (vk)
+            tma_load_4d(stg + (size_t)stage * a.stage_bytes + a.hstage_bytes, &tmap,
+                        &full[stage], (tx * kTileW - R) * 8, ty * kTileH - R, 0, p);
+          if (vsep) {
+          } else if (kbi < a.nkb0)
+            tma_load_4d(stg + (size_t)stage * a.stage_bytes, &tmap, &full[stage],
+                        (tx * kTileW - R) * EPG, ty * kTileH - R, a.in_goff + kbi * GPK, p);
+          else
+            tma_load_4d(stg + (size_t)stage * a.stage_bytes, &tmap1, &full[stage],
+                        (tx * kTileW - R) * EPG, ty * kTileH - R,
+                        a.in1_goff + (kbi - a.nkb0) * GPK, p);
         }
-      }
-      if (stop) break;
-      t += (two ? 2 : 1) * nctas;
-      if (two) {
-        ti = t1;
-        ti.next(a.step_dx, a.step_dy, a.step_dp, a.tiles_x, a.tiles_y);
-      } else {
-        ti = t1;
+        ++issued;
+        if (++stage == a.stages) { stage = 0; phase ^= 1; }
       }
     }
     griddep_launch();
@@ -461,8 +480,18 @@ __global__ void __launch_bounds__(conv_threads(KS, EPI, NCTA), 1) k_conv_tc(cons
       }
       mbar_wait_drain(wbar, 0);
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1) {
     // ---- MMA issuer ---------------------------------------------------------
+    // What bounds it: an M = 128 MMA takes 51 cycles of the tensor pipe for N
+    // = 64 (its A and B rows from shared memory), 66 for N = 128, 130 for N =
+    // 256, whatever the alignment of A's rows and with one accumulator as
+    // with two; so the issue must cost less than that. The whole warp runs
+    // the loop (its state then lives in uniform registers, which the MMA
+    // takes its descriptors from) and one elected lane issues; descriptors
+    // are 32-bit halves. By one thread with 64-bit descriptors and a second
+    // interleaved tile an MMA took 75 to 97 cycles to issue: per batch of 24,
+    // BF16 gates 11.0 -> 8.2 ms, BF16 conv 1 7.1 -> 6.5 ms, FP8 conv 1 4.8 ->
+    // 4.4 ms; the FP8 gates then wait for their epilogue.
     // All descriptor offsets are compile-time constants: one K-block is
     // taps x KB/16 MMAs whose descriptors differ from the block's base
     // descriptors by fixed amounts (addresses enter descriptors >> 4).
@@ -476,126 +505,108 @@ __global__ void __launch_bounds__(conv_threads(KS, EPI, NCTA), 1) k_conv_tc(cons
     bool ok = mbar_wait(wbar, 0, s_abort);
     int stage = 0, acc = 0;
     uint32_t phase = 0, aphase = 0;
-    // a.pairs: two tiles per round (the producer alternates their K-blocks,
-    // so two stages suffice), their MMAs interleaved into two accumulators so that
-    // consecutive MMAs never depend on each other's accumulator (the
-    // autotuner decides per shape class: faster for the FP8 3x3 convs,
-    // slower for the HBM-bound 1x1 convs)
-    const bool pairs = a.pairs && a.stages >= 2;
-    for (int t = cta; ok && t < a.tiles; t += (pairs ? 2 : 1) * nctas) {
-      const bool two = pairs && t + nctas < a.tiles;
-      const int acc1 = acc + 1 == kAcc ? 0 : acc + 1;
-      const uint32_t aphase1 = acc + 1 == kAcc ? aphase ^ 1 : aphase;
-      if (!mbar_wait(&acce[acc], aphase ^ 1, s_abort, 200)) break;
-      if (two && !mbar_wait(&acce[acc1], aphase1 ^ 1, s_abort, 200)) break;
-      fence_after();
-      const uint32_t d0 = tbase + (uint32_t)(acc * NCTA), d1 = tbase + (uint32_t)(acc1 * NCTA);
-      uint32_t accum = 0;
-      if constexpr (EPI == TE_HEADC) {
-        // a.nkb = 9 / a.tps stages per tile, a.tps taps per stage: A =
-        // 128 positions x KB channels per tap, rows of KB * element bytes
-        // (32, 64 or 128) swizzled like the TMA wrote them; each MMA takes
-        // the next 32 bytes of K within the rows
-        constexpr uint32_t rowb = KB * (F8 ? 1 : 2);
-        constexpr uint32_t swz = rowb == 128 ? 2u : rowb == 64 ? 4u : 6u;
-        const uint64_t b0 = sdesc(smem_u32(wsm), NCTA * 16u, 128u);
-        const uint32_t boxd = (128u * rowb) >> 4;   // descriptor step per tap
-        for (int kbi = 0; kbi < a.nkb; ++kbi) {
-          // stages of K-step kbi: the first tile's, then (paired) the second's
-          int s0 = stage + (two ? 2 * kbi : kbi);
-          uint32_t p0 = phase;
-          while (s0 >= a.stages) { s0 -= a.stages; p0 ^= 1; }
-          int s1 = s0 + 1;
-          uint32_t p1 = p0;
-          if (s1 >= a.stages) { s1 -= a.stages; p1 ^= 1; }
-          if (!mbar_wait(&full[s0], p0, s_abort)) { ok = false; break; }
-          if (two && !mbar_wait(&full[s1], p1, s_abort)) { ok = false; break; }
-          fence_after();
-          const uint64_t a0 = sdesc_sw(smem_u32(stg + (size_t)s0 * a.stage_bytes), 8u * rowb, swz);
-          const uint64_t a1 = sdesc_sw(smem_u32(stg + (size_t)s1 * a.stage_bytes), 8u * rowb, swz);
-          for (int tt = 0; tt < a.tps; ++tt) {
-            const int tap = kbi * a.tps + tt;
-#pragma unroll
-            for (int s = 0; s < KSTEPS; ++s) {
-              const uint32_t aoff = tt * boxd + ((32u * s) >> 4);
-              const uint32_t boff = ((uint32_t)(tap * GPK + 2 * s) * (NCTA * 16u)) >> 4;
-              if (F8) mma_fp8(d0, a0 + aoff, b0 + boff, idesc, accum);
-              else mma_bf16(d0, a0 + aoff, b0 + boff, idesc, accum);
-              if (two) {
-                if (F8) mma_fp8(d1, a1 + aoff, b0 + boff, idesc, accum);
-                else mma_bf16(d1, a1 + aoff, b0 + boff, idesc, accum);
-              }
-              accum = 1;
-            }
-          }
-          mma_commit(&empty[s0]);
-          if (two) mma_commit(&empty[s1]);
-        }
-      } else
-      for (int kbi = 0; kbi < a.nkb; ++kbi) {
-        // stages of this K-block: the first tile's, then (paired) the second's
-        int s0 = stage + (two ? 2 * kbi : kbi);
-        uint32_t p0 = phase;
-        while (s0 >= a.stages) { s0 -= a.stages; p0 ^= 1; }
-        int s1 = s0 + 1;
-        uint32_t p1 = p0;
-        if (s1 >= a.stages) { s1 -= a.stages; p1 ^= 1; }
-        if (!mbar_wait(&full[s0], p0, s_abort)) { ok = false; break; }
-        if (two && !mbar_wait(&full[s1], p1, s_abort)) { ok = false; break; }
+    const bool leader = elect_one();
+    // kEarly: the barriers of a K-block (its stage, and the accumulator when
+    // it starts a tile) are waited for before the last third of the MMAs of
+    // the block before it, so that the tensor pipe has work while they are
+    // polled (neither depends on the current block: its stage and its
+    // accumulator are others). It pays where the MMAs are the longer side
+    // (batch of 24, FP8 gates 4.76 -> 4.38 ms, BF16 conv 1 6.50 -> 6.26 ms);
+    // where the epilogue is, holding the tile's last MMAs back costs time (FP8
+    // conv 1 4.28 -> 4.45 ms, z conv 3.79 -> 4.07 ms).
+    constexpr bool kEarly = EPI == TE_LSTM || (KS == 3 && EPI == TE_STORE && !F8);
+    if (kEarly && ok && cta < a.tiles)
+      ok = mbar_wait(&acce[0], 1, s_abort, 200) && mbar_wait(&full[0], 0, s_abort);
+    for (int t = cta; ok && t < a.tiles; t += nctas) {
+      const uint32_t d = tbase + (uint32_t)(acc * NCTA);
+      if (!kEarly && !mbar_wait(&acce[acc], aphase ^ 1, s_abort, 200)) break;
+      for (int kbi = 0; ok && kbi < a.nkb; ++kbi) {
+        if (!kEarly && !mbar_wait(&full[stage], phase, s_abort)) { ok = false; break; }
         fence_after();
-        const uint64_t a0 = sdesc(smem_u32(stg + (size_t)s0 * a.stage_bytes), slab, HX * 16u);
-        const uint64_t a1 = sdesc(smem_u32(stg + (size_t)s1 * a.stage_bytes), slab, HX * 16u);
-        if (HV && kbi == 0) {
-          // v block (after the first K-block in the same stage, or alone
-          // in its stage): one BF16 MMA (K = 16, the block's two 16-byte
-          // groups) per tap, accumulating with the K-blocks' MMAs
-          const uint32_t idv = (1u << 4) | (1u << 7) | (1u << 10) |
-                               ((uint32_t)(NCTA >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-          const uint64_t bv = sdesc(smem_u32(wsm), NCTA * 16u, 128u);
-          const uint32_t vo = VMERGE ? a.hstage_bytes >> 4 : 0u;
-#pragma unroll
-          for (int tap = 0; tap < taps; ++tap) {
-            const uint32_t aoff = vo + (((uint32_t)((tap / KS) * HX + tap % KS) * 16u) >> 4);
-            const uint32_t boff = ((uint32_t)(tap * 2) * (NCTA * 16u)) >> 4;
-            mma_bf16(d0, a0 + aoff, bv + boff, idv, accum);
-            if (two) mma_bf16(d1, a1 + aoff, bv + boff, idv, accum);
-            accum = 1;
+        const uint32_t sb = smem_u32(stg) + (uint32_t)stage * a.stage_bytes;
+        const uint32_t wb = smem_u32(wsm);
+        const uint32_t first = kbi > 0 ? 1u : 0u;   // the tile's first MMA overwrites
+        const bool last = kbi + 1 == a.nkb;         // the tile's last K-block
+        uint64_t *const done = &empty[stage];
+        if (++stage == a.stages) { stage = 0; phase ^= 1; }
+        auto wait_next = [&]() {
+          if (!kEarly) return;
+          if (last) {
+            if (t + nctas >= a.tiles) return;
+            const int an = acc + 1 == kAcc ? 0 : acc + 1;
+            if (!mbar_wait(&acce[an], (an ? aphase : aphase ^ 1) ^ 1, s_abort, 200)) ok = false;
           }
-          if (!VMERGE) {
-            mma_commit(&empty[s0]);
-            if (two) mma_commit(&empty[s1]);
-            continue;
-          }
-        }
-        const int kh = kbi - (HV && !VMERGE ? 1 : 0);   // index in wt
-        const uint64_t b0 = sdesc(smem_u32(wsm) + a.wv_bytes + (uint32_t)kh * wblock, NCTA * 16u, 128u);
+          if (ok && !mbar_wait(&full[stage], phase, s_abort)) ok = false;
+        };
+        constexpr uint32_t bhi = sdesc_hi(128u);
+        if constexpr (EPI == TE_HEADC) {
+          // a.nkb = 9 / a.tps stages per tile, a.tps taps per stage: A =
+          // 128 positions x KB channels per tap, rows of KB * element bytes
+          // (32, 64 or 128) swizzled like the TMA wrote them; each MMA takes
+          // the next 32 bytes of K within the rows
+          constexpr uint32_t rowb = KB * (F8 ? 1 : 2);
+          constexpr uint32_t swz = rowb == 128 ? 2u : rowb == 64 ? 4u : 6u;
+          constexpr uint32_t boxd = (128u * rowb) >> 4;            // descriptor step per tap
+          constexpr uint32_t wtap = (GPK * NCTA * 16u) >> 4;       // and of the weights
+          constexpr uint32_t ahi = sdesc_hi(8u * rowb) | (swz << 29);
+          uint32_t ad = sdesc_lo(sb, 16u);
+          uint32_t bd = sdesc_lo(wb, NCTA * 16u) + (uint32_t)(kbi * a.tps) * wtap;
+          uint32_t accum = first;
+          for (int tt = 0; tt < a.tps; ++tt, ad += boxd, bd += wtap) {
+            if (leader) {
 #pragma unroll
-        for (int tap = 0; tap < taps; ++tap) {
-#pragma unroll
-          for (int s = 0; s < KSTEPS; ++s) {
-            const uint32_t aoff = ((uint32_t)(2 * s) * slab + (uint32_t)((tap / KS) * HX + tap % KS) * 16u) >> 4;
-            const uint32_t boff = ((uint32_t)(tap * GPK + 2 * s) * (NCTA * 16u)) >> 4;
-            if (F8) mma_fp8(d0, a0 + aoff, b0 + boff, idesc, accum);
-            else mma_bf16(d0, a0 + aoff, b0 + boff, idesc, accum);
-            if (two) {
-              if (F8) mma_fp8(d1, a1 + aoff, b0 + boff, idesc, accum);
-              else mma_bf16(d1, a1 + aoff, b0 + boff, idesc, accum);
+              for (int s = 0; s < KSTEPS; ++s) {
+                const uint32_t boff = ((uint32_t)(2 * s) * (NCTA * 16u)) >> 4;
+                mma_lo<F8>(d, ad + ((32u * s) >> 4), ahi, bd + boff, bhi, idesc,
+                           s > 0 ? 1u : accum);
+              }
             }
             accum = 1;
           }
+        } else {
+          const uint32_t ad = sdesc_lo(sb, slab);
+          constexpr uint32_t ahi = sdesc_hi(HX * 16u);
+          if (HV && kbi == 0 && leader) {
+            // v block (after the first K-block in the same stage, or alone
+            // in its stage): one BF16 MMA (K = 16, the block's two 16-byte
+            // groups) per tap, accumulating with the K-blocks' MMAs
+            constexpr uint32_t idv = (1u << 4) | (1u << 7) | (1u << 10) |
+                                     ((uint32_t)(NCTA >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+            const uint32_t av = ad + (VMERGE ? a.hstage_bytes >> 4 : 0u);
+            const uint32_t bv = sdesc_lo(wb, NCTA * 16u);
+#pragma unroll
+            for (int tap = 0; tap < taps; ++tap) {
+              const uint32_t aoff = ((uint32_t)((tap / KS) * HX + tap % KS) * 16u) >> 4;
+              const uint32_t boff = ((uint32_t)(tap * 2) * (NCTA * 16u)) >> 4;
+              mma_lo<false>(d, av + aoff, ahi, bv + boff, bhi, idv, tap > 0 ? 1u : 0u);
+            }
+          }
+          if (!HV || VMERGE || kbi > 0) {
+            const int kh = kbi - (HV && !VMERGE ? 1 : 0);   // index in wt
+            const uint32_t bd = sdesc_lo(wb + a.wv_bytes + (uint32_t)kh * wblock, NCTA * 16u);
+            constexpr int kAll = taps * KSTEPS, kHead = kAll * 2 / 3;
+            auto issue = [&](auto from, auto to) {
+#pragma unroll
+              for (int i = decltype(from)::value; i < decltype(to)::value; ++i) {
+                const int tap = i / KSTEPS, s = i % KSTEPS;
+                const uint32_t aoff = ((uint32_t)(2 * s) * slab +
+                                       (uint32_t)((tap / KS) * HX + tap % KS) * 16u) >> 4;
+                const uint32_t boff = ((uint32_t)(tap * GPK + 2 * s) * (NCTA * 16u)) >> 4;
+                mma_lo<F8>(d, ad + aoff, ahi, bd + boff, bhi, idesc, i > 0 || HV ? 1u : first);
+              }
+            };
+            using std::integral_constant;
+            if (leader) issue(integral_constant<int, 0>(), integral_constant<int, kHead>());
+            wait_next();
+            if (leader) issue(integral_constant<int, kHead>(), integral_constant<int, kAll>());
+          }
         }
-        mma_commit(&empty[s0]);
-        if (two) mma_commit(&empty[s1]);
+        if (leader) mma_commit(done);
       }
-      if (!ok) break;
-      mma_commit(&accf[acc]);
-      if (two) mma_commit(&accf[acc1]);
-      // advance past the consumed stages and accumulators
-      const int used = (two ? 2 : 1) * a.nkb;
-      stage += used;
-      while (stage >= a.stages) { stage -= a.stages; phase ^= 1; }
-      acc += two ? 2 : 1;
-      if (acc >= kAcc) { acc -= kAcc; aphase ^= 1; }
+      if (!kEarly && !ok) break;
+      // (an expired early wait is for the next block)
+      if (leader) mma_commit(&accf[acc]);
+      if (++acc == kAcc) { acc = 0; aphase ^= 1; }
     }
   } else if (warp >= 2) {
     // ---- epilogue: warps 2 .. 2 + EW - 1; warp w reads TMEM lanes
@@ -643,11 +654,12 @@ __global__ void __launch_bounds__(conv_threads(KS, EPI, NCTA), 1) k_conv_tc(cons
       const int64_t pix = (int64_t)y * a.W + x;
       if (EPI == TE_LSTM) {
         const int Hp = a.H >> a.up, Wp = a.W >> a.up;
-        const int64_t ppix = ((int64_t)p * Hp + (y >> a.up)) * Wp + (x >> a.up);
+        const int64_t ppix = (int64_t)(y >> a.up) * Wp + (x >> a.up);
 #pragma unroll
         for (int k = 0; k < NCP; ++k)
           cpo[k] = a.first ? make_uint4(0u, 0u, 0u, 0u)
-                           : __ldg(reinterpret_cast<const uint4 *>(a.c_prev + ppix * a.C + n0 / 4 + 8 * k));
+                           : __ldg(reinterpret_cast<const uint4 *>(a.c_prev) +
+                                   ((int64_t)p * (a.C >> 3) + (n0 >> 5) + k) * Hp * Wp + ppix);
       } else if (HEADK || (STORE && a.res)) {
         const bool need = STORE ||
                           (a.compact_n ? pix < a.compact_n : step_of(y, x) == a.step);
@@ -827,18 +839,22 @@ __global__ void __launch_bounds__(conv_threads(KS, EPI, NCTA), 1) k_conv_tc(cons
         }
 #pragma unroll
         for (int k = 0; k < NH / 4; k += 8)
-          store_bf16x8(a.c_new + ((int64_t)p * hw + pix) * a.C + ch0 + k, cn + k);
+          store_bf16x8(a.c_new + (((int64_t)p * (a.C >> 3) + ((ch0 + k) >> 3)) * hw + pix) * 8,
+                       cn + k);
 #pragma unroll
         for (int g = 0; g < NH / 32; ++g)
           store_bf16x8(a.out + (((int64_t)p * G + a.out_goff + (ch0 >> 3) + g) * hw + pix) * 8,
                        hv + 8 * g);
-        if (NH % 64 == 0 && a.out8) {
+        if (a.out8) {
+          // 8 channels (half of a 16-byte group) at a time
 #pragma unroll
-          for (int g = 0; g < NH / 64; ++g) {
-            float f[16];
+          for (int k = 0; k < NH / 4; k += 8) {
+            float f[8];
 #pragma unroll
-            for (int e = 0; e < 16; ++e) f[e] = hv[16 * g + e] * s_osc[col0 / 4 + 16 * g + e];
-            store_fp8x16(a.out8 + (((int64_t)p * a.out8_G16 + (ch0 >> 4) + g) * hw + pix) * 16, f);
+            for (int e = 0; e < 8; ++e) f[e] = hv[k + e] * s_osc[col0 / 4 + k + e];
+            store_fp8x8(a.out8 + (((int64_t)p * a.out8_G16 + ((ch0 + k) >> 4)) * hw + pix) * 16 +
+                            ((ch0 + k) & 8),
+                        f);
           }
         }
       } else {  // TE_HEAD: z' = res + acc + b over all C columns, then 1x1(C->2)
@@ -1131,23 +1147,22 @@ static bool headc_ok(int h, int w) { return h >= 4 && w >= 8; }
 
 
 // ---- autotuner -------------------------------------------------------------
-// Per (kernel variant, size class = log2 of the tile count) the MMA issue
-// schedule: one or two tiles per round. The candidates are sampled in place,
-// round robin, on the real launches of the decode / encode pipeline (each
+// Per (kernel variant, size class = log2 of the tile count) the pipeline
+// shape. The candidates are sampled in place, round robin, on the real
+// launches of the decode / encode pipeline (each
 // launch bracketed by events that are read back later without a
 // synchronisation), so that the choice reflects the caches and concurrency
 // the kernel really sees; after kSamples samples of every candidate the
 // fastest median wins (the median ignores a one-off outlier such as the
 // first launch of a kernel, which loads its module). Results do not depend
 // on the schedule.
-// Candidates: bit 0 = paired MMA issue, bit 1 = the alternative pipeline
-// shape (a shallower pipeline for the plain convolutions, the second-best
-// tile shape for the compact head).
+// Candidates: bit 1 = the alternative pipeline shape (a shallower pipeline
+// for the plain convolutions, the second-best tile shape for the compact
+// head); bit 0 is not used (reported as not sampled).
 constexpr int kTuneCand = 4, kSamples = 3;
 struct TuneChoice {
-  int pairs = 0;
   int shape = 0;
-  int cand() const { return pairs | (shape << 1); }
+  int cand() const { return shape << 1; }
 };
 struct TuneEntry {
   bool tuned = false;
@@ -1204,7 +1219,6 @@ static void tune_poll_locked() {
         for (int c = 0; c < kTuneCand; ++c)
           if (t.n[c] && t.median(c) < best) {
             best = t.median(c);
-            t.choice.pairs = c & 1;
             t.choice.shape = c >> 1;
           }
         t.tuned = true;
@@ -1220,16 +1234,14 @@ static void tune_poll_locked() {
 
 // The schedule of the next launch of a class. While the class is being tuned
 // (sample = true) the launch is a sample of candidate `cand`.
-static TuneChoice tune_next(uint64_t key, bool can_pair, bool has_alt, cudaStream_t st,
-                            bool &sample, int &cand) {
-  TuneChoice c;
-  c.pairs = ((key >> 32) & 0xFF) == 3 && ((key >> 9) & 1) && can_pair;  // default
+static TuneChoice tune_next(uint64_t key, bool has_alt, cudaStream_t st, bool &sample,
+                            int &cand) {
+  TuneChoice c;   // the default shape
   sample = false;
   std::lock_guard<std::mutex> lk(g_tune_mu);
   tune_poll_locked();
   TuneEntry &t = g_tune[key];
   if (t.tuned) {
-    c.pairs = t.choice.pairs && can_pair;
     c.shape = t.choice.shape && has_alt;
     return c;
   }
@@ -1240,20 +1252,17 @@ static TuneChoice tune_next(uint64_t key, bool can_pair, bool has_alt, cudaStrea
     cudaGetLastError();
     return c;
   }
-  auto valid = [&](int k) { return (!(k & 1) || can_pair) && (!(k & 2) || has_alt); };
-  int nvalid = 0;
-  for (int k = 0; k < kTuneCand; ++k) nvalid += valid(k) ? 1 : 0;
-  if (nvalid == 1) {  // nothing to choose
+  if (!has_alt) {  // nothing to choose
     t.tuned = true;
     t.choice = TuneChoice{};
     return c;
   }
+  auto valid = [](int k) { return !(k & 1); };
   while (!valid(t.next)) t.next = (t.next + 1) % kTuneCand;
   cand = t.next;
   if (t.issued[cand] >= kSamples) return c;  // enough in flight; wait for read-back
   do { t.next = (t.next + 1) % kTuneCand; } while (!valid(t.next));
   t.issued[cand] += 1;
-  c.pairs = cand & 1;
   c.shape = cand >> 1;
   sample = true;
   return c;
@@ -1276,9 +1285,8 @@ int tune_set_enabled(int on) {
   return old;
 }
 // One line per tuned class: "ks kb ncta epi f8 log2tiles choice t0 t1 t2 t3"
-// (choice = the kept candidate, bit 0 paired issue, bit 1 alternative
-// pipeline shape; t = median sampled time of each candidate in microseconds,
-// -1 = not sampled).
+// (choice = the kept candidate, bit 1 = alternative pipeline shape; t = median
+// sampled time of each candidate in microseconds, -1 = not sampled).
 std::string tune_report() {
   std::lock_guard<std::mutex> lk(g_tune_mu);
   tune_poll_locked();
@@ -1412,8 +1420,7 @@ static int conv_tc(pw_ctx *ctx, const TcWeights::Conv &cv, const void *in, int i
   const uint64_t key = tune_key(cv, a.epi, a.tiles);
   bool sample = false;
   int cand = 0;
-  const TuneChoice ch = tune_next(key, true, has_alt, ctx->stream, sample, cand);
-  a.pairs = ch.pairs;
+  const TuneChoice ch = tune_next(key, has_alt, ctx->stream, sample, cand);
   if (ch.shape && hc) set_hc_shape(lj_alt);
   a.stages = (ch.shape && !hc) ? st_alt : st_def;
   const size_t smem = fixed + (size_t)a.stages * a.stage_bytes;

@@ -95,13 +95,16 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t addr, uint32_t lbo, uint32_t 
   return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)((lbo >> 4) & 0x3FFFu) << 16) |
          ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46);
 }
-// Swizzled K-major descriptor (mode 2 = 128-byte, 4 = 64-byte, 6 = 32-byte
-// swizzle; rows of that many bytes, 8-row groups sbo bytes apart; the
-// leading offset is unused)
-__device__ __forceinline__ uint64_t sdesc_sw(uint32_t addr, uint32_t sbo, uint32_t mode) {
-  return (uint64_t)((addr & 0x3FFFFu) >> 4) | (1ull << 16) |
-         ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46) | ((uint64_t)mode << 61);
+// Its halves: address and leading offset, stride offset and constants.
+__host__ __device__ __forceinline__ constexpr uint32_t sdesc_lo(uint32_t addr, uint32_t lbo) {
+  return ((addr & 0x3FFFFu) >> 4) | (((lbo >> 4) & 0x3FFFu) << 16);
 }
+__host__ __device__ __forceinline__ constexpr uint32_t sdesc_hi(uint32_t sbo) {
+  return ((sbo >> 4) & 0x3FFFu) | (1u << 14);
+}
+// (Swizzled K-major descriptors: mode 2 = 128-byte, 4 = 64-byte, 6 = 32-byte
+// swizzle in bits 29..31 of the high half; rows of that many bytes, 8-row
+// groups sbo bytes apart; leading offset 16, unused.)
 __device__ __forceinline__ void mma_bf16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc,
                                          uint32_t accum) {
   asm volatile(
