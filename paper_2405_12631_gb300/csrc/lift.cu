@@ -322,12 +322,13 @@ struct LiftTcSmem {
   alignas(128) __nv_bfloat16 w3[9 * 2 * LF * 8];
   alignas(16) float in[LI * LI];
   alignas(16) float rout[LT * LT];
-  alignas(16) float w1t[9 * LF];
-  alignas(16) float b1[LF];
-  alignas(16) float b2[LF];
   alignas(8) uint64_t bar;
   uint32_t tmem;
-  float b3;
+};
+// The FP32 weights of a step as a kernel parameter: w1 [tap][c], the biases.
+struct LiftTcWt {
+  alignas(16) float w1[9 * LF];
+  float b1[LF], b2[LF], b3;
 };
 
 // Bounded wait of every thread for completion phase `parity` of the MMA
@@ -350,8 +351,11 @@ __device__ __forceinline__ bool lift_mma_wait(uint64_t *bar, uint32_t parity) {
 }
 
 // (six resident CTAs per SM: 40 registers instead of 48, which allowed five;
-// lifting class 4.50 -> 4.45 ms per batch of 24)
-__global__ void __launch_bounds__(256, 6) k_lift_tc(LiftStepParams a) {
+// lifting class 4.50 -> 4.45 ms per batch of 24. Layer 1 from the parameter
+// bank and on its 400 positions only: 4.36 -> 3.51 ms; what bounds it now is
+// issue, 64 % of the slots.)
+__global__ void __launch_bounds__(256, 6) k_lift_tc(const __grid_constant__ LiftStepParams a,
+                                                    const __grid_constant__ LiftTcWt wt) {
   extern __shared__ __align__(1024) uint8_t lsm_raw[];
   LiftTcSmem &S = *reinterpret_cast<LiftTcSmem *>(lsm_raw);
   __nv_bfloat16 *const a2 = S.a1;   // layer-2 slab over the consumed layer-1 slab
@@ -380,10 +384,6 @@ __global__ void __launch_bounds__(256, 6) k_lift_tc(LiftStepParams a) {
     const int yy = y0 + e / LI - 3, xx = x0 + e % LI - 3;
     S.in[e] = (yy >= 0 && yy < H && xx >= 0 && xx < W) ? acc_get(a.src, p, yy, xx) : 0.f;
   }
-  for (int e = t; e < LF * 9; e += 256) {
-    const int c = e / 9, tap = e % 9;  // source [c][tap]
-    S.w1t[tap * LF + c] = a.net.w1[e];
-  }
   {
     // the packed B operands of layers 2 and 3 (9 x 2 x 16 x 8 BF16 each)
     constexpr int kB16 = 9 * 2 * LF * 8 * 2 / 16;
@@ -394,8 +394,6 @@ __global__ void __launch_bounds__(256, 6) k_lift_tc(LiftStepParams a) {
       reinterpret_cast<uint4 *>(S.w3)[i] = __ldg(src3 + i);
     }
   }
-  if (t < LF) { S.b1[t] = a.net.b1[t]; S.b2[t] = a.net.b2[t]; }
-  if (t == 0) S.b3 = a.net.b3[0];
   fence_before();
   __syncthreads();
   fence_after();
@@ -403,39 +401,40 @@ __global__ void __launch_bounds__(256, 6) k_lift_tc(LiftStepParams a) {
   const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(LF >> 3) << 17) |
                          ((uint32_t)(128 >> 4) << 24);
 
-  // layer 1 on the 20 x 24 region (origin y0 - 2, x0 - 2), one position and
-  // one group of 8 channels per item; padding positions are written as 0
-  for (int it = t; it < 2 * kA; it += 256) {
-    const int pos = it >> 1, g = it & 1;
-    const int r = pos / kRS, c = pos % kRS;
+  // layer 1 on the 20 x 20 region (origin y0 - 2, x0 - 2), one position per
+  // item. (The slab's padding stays as it is: an MMA row reads the rows of
+  // its own taps only, and rows that read padding are not used.) The weights
+  // come from the parameter bank: as broadcast loads from shared memory they
+  // had its port at 86 %, the bound of this kernel.
+  for (int it = t; it < L1 * L1; it += 256) {
+    const int r = it / L1, c = it % L1, pos = r * kRS + c;
     const int yy = y0 - 2 + r, xx = x0 - 2 + c;
-    float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if (r < L1 && c < L1 && yy >= 0 && yy < H && xx >= 0 && xx < W) {
+    const bool inside = yy >= 0 && yy < H && xx >= 0 && xx < W;
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
       // channel pairs in packed FP32 FMAs (the same rounding as fmaf)
       uint64_t acc[4];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) acc[k] = f2pack(S.b1[8 * g + 2 * k], S.b1[8 * g + 2 * k + 1]);
+      for (int k = 0; k < 4; ++k) acc[k] = f2pack(wt.b1[8 * g + 2 * k], wt.b1[8 * g + 2 * k + 1]);
 #pragma unroll
       for (int tap = 0; tap < 9; ++tap) {
         const float iv = S.in[(r + tap / 3) * LI + c + tap % 3];
         const uint64_t iv2 = f2pack(iv, iv);
-        const float4 wa = *reinterpret_cast<const float4 *>(S.w1t + tap * LF + 8 * g);
-        const float4 wb = *reinterpret_cast<const float4 *>(S.w1t + tap * LF + 8 * g + 4);
-        acc[0] = fma2(f2pack(wa.x, wa.y), iv2, acc[0]);
-        acc[1] = fma2(f2pack(wa.z, wa.w), iv2, acc[1]);
-        acc[2] = fma2(f2pack(wb.x, wb.y), iv2, acc[2]);
-        acc[3] = fma2(f2pack(wb.z, wb.w), iv2, acc[3]);
+        const uint64_t *w = reinterpret_cast<const uint64_t *>(wt.w1 + tap * LF + 8 * g);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) acc[k] = fma2(w[k], iv2, acc[k]);
       }
+      __align__(16) __nv_bfloat16 hb[8];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) f2unpack(acc[k], v[2 * k], v[2 * k + 1]);
-#pragma unroll
-      for (int k = 0; k < 8; ++k) v[k] = tanh_fast(v[k]);
+      for (int k = 0; k < 4; ++k) {
+        float lo, hi;
+        f2unpack(acc[k], lo, hi);
+        hb[2 * k] = __float2bfloat16_rn(inside ? tanh_fast(lo) : 0.f);
+        hb[2 * k + 1] = __float2bfloat16_rn(inside ? tanh_fast(hi) : 0.f);
+      }
+      *reinterpret_cast<uint4 *>(S.a1 + ((size_t)g * kA + pos) * 8) =
+          *reinterpret_cast<const uint4 *>(hb);
     }
-    __align__(16) __nv_bfloat16 hb[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) hb[k] = __float2bfloat16_rn(v[k]);
-    *reinterpret_cast<uint4 *>(S.a1 + ((size_t)g * kA + pos) * 8) =
-        *reinterpret_cast<const uint4 *>(hb);
   }
   fence_proxy_async();
   __syncthreads();
@@ -475,7 +474,7 @@ __global__ void __launch_bounds__(256, 6) k_lift_tc(LiftStepParams a) {
         __align__(16) __nv_bfloat16 hb[LF];
 #pragma unroll
         for (int k = 0; k < LF; ++k)
-          hb[k] = __float2bfloat16_rn(live ? tanh_fast(v[k] + S.b2[k]) : 0.f);
+          hb[k] = __float2bfloat16_rn(live ? tanh_fast(v[k] + wt.b2[k]) : 0.f);
         *reinterpret_cast<uint4 *>(a2 + (size_t)m * 8) = *reinterpret_cast<const uint4 *>(hb);
         *reinterpret_cast<uint4 *>(a2 + ((size_t)kA2 + m) * 8) =
             *reinterpret_cast<const uint4 *>(hb + 8);
@@ -512,7 +511,7 @@ __global__ void __launch_bounds__(256, 6) k_lift_tc(LiftStepParams a) {
       tmem_ld16(tbase + ((uint32_t)(32 * q) << 16) + (uint32_t)(i * LF), v);
       const int m = i * 128 + 32 * q + lane;
       const int r = m / kRS, c = m % kRS;
-      if (r < LT && c < LT) S.rout[r * LT + c] = v[0] + S.b3;
+      if (r < LT && c < LT) S.rout[r * LT + c] = v[0] + wt.b3;
     }
   }
   fence_before();
@@ -647,7 +646,12 @@ void launch_lift_step(const LiftStepParams &a, cudaStream_t st) {
     });
     const int tiles = ((a.H + LT - 1) / LT) * ((a.W + LT - 1) / LT);
     dim3 grid(tiles, 1, a.P);
-    k_lift_tc<<<grid, 256, sizeof(LiftTcSmem) + 1024, st>>>(a);
+    LiftTcWt wt;
+    std::memcpy(wt.w1, a.net.wt_host, sizeof(wt.w1));
+    std::memcpy(wt.b1, a.net.wt_host + 288, sizeof(wt.b1));
+    std::memcpy(wt.b2, a.net.wt_host + 304, sizeof(wt.b2));
+    wt.b3 = a.net.wt_host[320];
+    k_lift_tc<<<grid, 256, sizeof(LiftTcSmem) + 1024, st>>>(a, wt);
     return;
   }
   // large tiles where they fill the chip, small ones (a quarter of the work
