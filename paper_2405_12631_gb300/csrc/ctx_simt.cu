@@ -18,6 +18,9 @@
 #include "ctx_kernels.cuh"
 #include "f32x2.cuh"
 
+#include <algorithm>
+#include <atomic>
+
 namespace pw {
 
 __device__ __forceinline__ float sigm(float x) { return 1.f / (1.f + expf(-x)); }
@@ -49,102 +52,185 @@ __device__ __forceinline__ long long hsig_i(long long x) {
 }
 __device__ __forceinline__ long long htanh_i(long long x) { return clamp_ll(8 * x, 128); }
 
-// Generic NHWC convolution, KS x KS (KS = 1 or 3, zero padding), output
-// channels [blockIdx.y * CO_T, +CO_T). Tile: 8 rows x 16 columns of one
-// plane (blockIdx.z); 256 threads, each 4 consecutive pixels x CO_T/8
-// channels. Weights are [KS*KS][cin][cout_total].
-template <int KS, int CO_T, int EPI>
-__global__ void __launch_bounds__(256) k_conv_simt(ConvParams a) {
-  constexpr int TH = 8, TW = 16, CI = (CO_T >= 128 ? 4 : 8), R = KS / 2;
-  constexpr int HH = TH + KS - 1, HW = TW + KS - 1;
-  constexpr int NC = CO_T / 8;
-  // input tile, one plane per channel; the plane stride avoids shared-memory
-  // bank conflicts of the channel-fastest fill below
-  constexpr int PS = HH * HW + ((HH * HW) % 32 == 0 ? 4 : 0);
-  __shared__ float s_in[CI * PS];
-  __shared__ __align__(16) float s_w[KS * KS][CI][CO_T];
-  __shared__ float s_head[EPI == EPI_HEAD ? 8 : 1][TH * TW][2];
+// 16 bytes from global to shared memory, asynchronously; zeros when !valid.
+__device__ __forceinline__ void cp16(void *dst, const void *src, bool valid) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(src), "r"(valid ? 16 : 0)
+               : "memory");
+}
 
+// Generic NHWC convolution, KS x KS (KS = 1 or 3, zero padding). A block
+// computes a tile of 32 PX positions of one plane (blockIdx.z) x WG NC output
+// channels from blockIdx.y WG NC on: warp w has channels w NC .. + NC - 1, a
+// lane PX positions. Weights are [KS*KS][cin][cout_total].
+//
+// EPI_HEAD computes the step's own positions only (a quarter of the plane;
+// nothing else is used): TH rows x TW positions of a row, x = phase + 4 j,
+// the phase by the row's parity.
+//
+// What bounds it: on large planes the loads from shared memory (a thread
+// reads PX + NC values for PX NC multiply-adds, and the port returns one
+// register of a warp per cycle), on small ones the latency of a block. So the
+// input tile and the weights stream through a ring of kStages stages of CK
+// input channels by 16-byte asynchronous copies (one barrier per stage, no
+// load is waited for while another could run); the input lies in planes of 4
+// channels, 16 bytes per position, which lanes read side by side (for the
+// head columns are split by x mod 4, so that a step's positions are
+// neighbours too); and a plane with few tiles is split into more and smaller
+// blocks (see the launcher). Measured with C = 32, 3x3 32 -> 32 / gates / head
+// / 1x1: 24 x 32 plane 23 / 58 / 24 / 10..18 us -> 8 / 13 / 8 / 4 us; 192 x 256
+// plane 39 / 240 / 41 / 22 us -> 34 / 181 / 18 / 14..20 us (against four chunks
+// of synchronous 4-byte loads, and the head at every position).
+//
+// Every output is one chain in a fixed order: chunks of 8 input channels (4
+// for the head of 128), within a chunk tap by tap, channel by channel.
+template <int KS, int WG, int NC, int PX, int EPI>
+struct SimtCfg {
+  static constexpr int CO = WG * NC;
+  static constexpr int TW = PX == 4 ? 16 : 8, TH = 32 * PX / TW;
+  static constexpr bool kStep = EPI == EPI_HEAD;
+  static constexpr int HH = TH + KS - 1;                       // rows staged
+  static constexpr int HW = kStep ? 4 * (TW + 1) : TW + KS - 1;   // slots per row
+  static constexpr int HP = HH * HW;
+  // input channels per stage
+  static constexpr int CK = KS == 1 ? (kStep ? 16 : 32) : (NC == 16 ? 4 : 8);
+  static constexpr int kStages = 3;
+  static constexpr int kInF = CK * HP, kWF = KS * KS * CK * CO;   // floats of a stage
+  static constexpr int kHead = kStep ? 8 * TH * TW * 2 : 0;
+  static constexpr int kSmem = (kStages * (kInF + kWF) + kHead) * 4;
+};
+template <int KS, int WG, int NC, int PX, int EPI>
+__global__ void __launch_bounds__(32 * WG) k_conv_simt(const __grid_constant__ ConvParams a) {
+  using G = SimtCfg<KS, WG, NC, PX, EPI>;
+  constexpr int R = KS / 2, NT = 32 * WG, CK = G::CK;
+  extern __shared__ __align__(16) float sm_conv[];
   const int t = threadIdx.x;
-  const int pg = t & 31, cg = t >> 5;
-  const int prow = pg >> 2, pcol = (pg & 3) * 4;
+  const int lane = t & 31, cg = t >> 5;
   const int p = blockIdx.z;
-  const int tiles_x = (a.W + TW - 1) / TW;
-  const int y0 = (blockIdx.x / tiles_x) * TH, x0 = (blockIdx.x % tiles_x) * TW;
-  const int co0 = blockIdx.y * CO_T;
+  // tile origin: row y0, column x0 (head: position j0 of a row)
+  const int npos = G::kStep ? max(row_count(a.W, step_phase(a.step, 0)),
+                                  row_count(a.W, step_phase(a.step, 1)))
+                            : a.W;
+  const int tiles_x = (npos + G::TW - 1) / G::TW;
+  const int y0 = (blockIdx.x / tiles_x) * G::TH, x0 = (blockIdx.x % tiles_x) * G::TW;
+  const int co0 = blockIdx.y * G::CO;
   const float *inp = a.in + (int64_t)p * a.H * a.W * a.in_cs + a.in_co;
 
-  // accumulators of output channels (2k, 2k + 1) of pixel i in one packed
-  // FP32 pair: each element takes the same fused multiply-adds in the same
-  // order as a scalar accumulator (bit-identical results, half the
-  // instructions)
-  uint64_t accp[4][NC / 2];
+  const int nchunk = a.cin / CK;
+  auto stage_in = [&](int k) { return sm_conv + (k % G::kStages) * (G::kInF + G::kWF); };
+  auto load = [&](int k) {
+    float *si = stage_in(k), *sw = si + G::kInF;
+    const int c0 = k * CK;
+    for (int e = t; e < (CK / 4) * G::HP; e += NT) {
+      const int g = e % (CK / 4), q = e / (CK / 4);
+      const int r = q / G::HW, u = q % G::HW;
+      // head: columns 4 x0 - 1 + u, stored as (u mod 4, u / 4)
+      const int yy = y0 + r - R, xx = G::kStep ? 4 * x0 - 1 + u : x0 + u - R;
+      const bool in = yy >= 0 && yy < a.H && xx >= 0 && xx < a.W;
+      const int slot = G::kStep ? (u & 3) * (G::TW + 1) + (u >> 2) : u;
+      cp16(si + (g * G::HP + r * G::HW + slot) * 4,
+           inp + (in ? ((int64_t)yy * a.W + xx) * a.in_cs + c0 + 4 * g : 0), in);
+    }
+    for (int e = t; e < KS * KS * CK * (G::CO / 4); e += NT) {
+      const int j = e % (G::CO / 4), row = e / (G::CO / 4);   // row = tap * CK + c
+      const int tap = row / CK, c = row % CK;
+      cp16(sw + row * G::CO + 4 * j,
+           a.w + ((int64_t)tap * a.cin + c0 + c) * a.cout_total + co0 + 4 * j, true);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+
+  // positions of this lane: (ty[i], tx[i]) in the tile, slot of tap column dx
+  int base[PX], dxo[PX][KS];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < PX; ++i) {
+    const int q = lane + 32 * i, ty = q / G::TW, tx = q % G::TW;
+    base[i] = ty * G::HW + tx;
+#pragma unroll
+    for (int dx = 0; dx < KS; ++dx) {
+      if (G::kStep) {
+        const int v = step_phase(a.step, (y0 + ty) & 1) + dx + (KS == 1 ? 1 : 0);
+        dxo[i][dx] = (v & 3) * (G::TW + 1) + (v >> 2);
+      } else {
+        dxo[i][dx] = dx;
+      }
+    }
+  }
+  // accumulators of output channels (2k, 2k + 1) of a position in one packed
+  // FP32 pair: each element takes the same fused multiply-adds in the same
+  // order as a scalar accumulator
+  uint64_t accp[PX][NC / 2];
+#pragma unroll
+  for (int i = 0; i < PX; ++i)
 #pragma unroll
     for (int k = 0; k < NC / 2; ++k) accp[i][k] = 0ull;
 
-  for (int c0 = 0; c0 < a.cin; c0 += CI) {
-    __syncthreads();
-    // channel fastest: consecutive threads read a pixel's consecutive
-    // channels (one 32-byte sector per pixel for CI = 8)
-    for (int e = t; e < CI * HH * HW; e += 256) {
-      const int c = e % CI, r = e / CI;
-      const int yy = y0 + r / HW - R, xx = x0 + r % HW - R;
-      float v = 0.f;
-      if (c0 + c < a.cin && yy >= 0 && yy < a.H && xx >= 0 && xx < a.W)
-        v = inp[((int64_t)yy * a.W + xx) * a.in_cs + c0 + c];
-      s_in[c * PS + r] = v;
-    }
-    for (int e = t; e < KS * KS * CI * CO_T; e += 256) {
-      int tap = e / (CI * CO_T), r = e % (CI * CO_T);
-      int c = r / CO_T, o = r % CO_T;
-      float v = 0.f;
-      if (c0 + c < a.cin && co0 + o < a.cout_total)
-        v = a.w[((int64_t)tap * a.cin + c0 + c) * a.cout_total + co0 + o];
-      s_w[tap][c][o] = v;
-    }
-    __syncthreads();
+#pragma unroll
+  for (int k = 0; k < G::kStages - 1; ++k) {
+    if (k < nchunk) load(k);
+    else asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  for (int k = 0; k < nchunk; ++k) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(G::kStages - 2) : "memory");
+    __syncthreads();   // chunk k landed; chunk k - 1 is consumed
+    if (k + G::kStages - 1 < nchunk) load(k + G::kStages - 1);
+    else asm volatile("cp.async.commit_group;" ::: "memory");
+    const float4 *si = reinterpret_cast<const float4 *>(stage_in(k));
+    const float *sw = stage_in(k) + G::kInF + cg * NC;
 #pragma unroll
     for (int tap = 0; tap < KS * KS; ++tap) {
       const int dy = tap / KS, dx = tap % KS;
 #pragma unroll
-      for (int c = 0; c < CI; ++c) {
-        float xv[4];
+      for (int g = 0; g < CK / 4; ++g) {
+        float xv[PX][4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) xv[i] = s_in[c * PS + (prow + dy) * HW + pcol + i + dx];
-        const uint64_t *wrow = reinterpret_cast<const uint64_t *>(&s_w[tap][c][cg * NC]);
-        uint64_t wp[NC / 2];
+        for (int i = 0; i < PX; ++i) {
+          const float4 f = si[g * G::HP + base[i] + dy * G::HW + dxo[i][dx]];
+          xv[i][0] = f.x; xv[i][1] = f.y; xv[i][2] = f.z; xv[i][3] = f.w;
+        }
 #pragma unroll
-        for (int k = 0; k < NC / 2; ++k) wp[k] = wrow[k];
+        for (int e = 0; e < 4; ++e) {
+          const ulonglong2 *wrow =
+              reinterpret_cast<const ulonglong2 *>(sw + (tap * CK + 4 * g + e) * G::CO);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const uint64_t xx = f2pack(xv[i], xv[i]);
+          for (int k2 = 0; k2 < NC / 4; ++k2) {
+            const ulonglong2 w2 = wrow[k2];
 #pragma unroll
-          for (int k = 0; k < NC / 2; ++k) accp[i][k] = fma2(wp[k], xx, accp[i][k]);
+            for (int i = 0; i < PX; ++i) {
+              const uint64_t xx = f2pack(xv[i][e], xv[i][e]);
+              accp[i][2 * k2] = fma2(w2.x, xx, accp[i][2 * k2]);
+              accp[i][2 * k2 + 1] = fma2(w2.y, xx, accp[i][2 * k2 + 1]);
+            }
+          }
         }
       }
     }
   }
-  float acc[4][NC];
+  float acc[PX][NC];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < PX; ++i)
 #pragma unroll
     for (int k = 0; k < NC / 2; ++k) f2unpack(accp[i][k], acc[i][2 * k], acc[i][2 * k + 1]);
 
-  const int y = y0 + prow;
-  if (EPI == EPI_STORE) {
+  // plane position of this lane's i-th position
+  auto pos = [&](int q, int &y, int &x) {
+    const int ty = q / G::TW, tx = q % G::TW;
+    y = y0 + ty;
+    x = G::kStep ? step_phase(a.step, y & 1) + 4 * (x0 + tx) : x0 + tx;
+  };
+  if constexpr (EPI == EPI_STORE) {
     // four channels per 16-byte access (channel counts are multiples of
     // 32, channel offsets and row strides multiples of 4 floats)
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int x = x0 + pcol + i;
+    for (int i = 0; i < PX; ++i) {
+      int y, x;
+      pos(lane + 32 * i, y, x);
       if (y >= a.H || x >= a.W) continue;
       const int64_t pix = ((int64_t)p * a.H + y) * a.W + x;
 #pragma unroll
       for (int j = 0; j < NC; j += 4) {
         const int co = co0 + cg * NC + j;
-        if (co >= a.cout_total) continue;
         const float4 bb = *reinterpret_cast<const float4 *>(a.b + co);
         float v[4] = {acc[i][j] + bb.x, acc[i][j + 1] + bb.y, acc[i][j + 2] + bb.z,
                       acc[i][j + 3] + bb.w};
@@ -170,11 +256,12 @@ __global__ void __launch_bounds__(256) k_conv_simt(ConvParams a) {
             make_float4(v[0], v[1], v[2], v[3]);
       }
     }
-  } else if (EPI == EPI_LSTM) {
+  } else if constexpr (EPI == EPI_LSTM) {
     // output channel o = 4 * ch + gate (gate order i, f, o, g)
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int x = x0 + pcol + i;
+    for (int i = 0; i < PX; ++i) {
+      int y, x;
+      pos(lane + 32 * i, y, x);
       if (y >= a.H || x >= a.W) continue;
       const int64_t pix = ((int64_t)p * a.H + y) * a.W + x;
       const int Hp = a.H >> a.up, Wp = a.W >> a.up;
@@ -206,15 +293,16 @@ __global__ void __launch_bounds__(256) k_conv_simt(ConvParams a) {
       }
     }
   } else {  // EPI_HEAD: z' = res + acc + b over all C channels, then 1x1(C->2)
-    float pm[4], pr[4];
+    static_assert(WG == 8, "the head's partial sums are those of 8 channel groups");
+    float(*s_head)[G::TH * G::TW][2] = reinterpret_cast<float(*)[G::TH * G::TW][2]>(
+        sm_conv + G::kStages * (G::kInF + G::kWF));
 #pragma unroll
-    for (int i = 0; i < 4; ++i) { pm[i] = 0.f; pr[i] = 0.f; }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int x = x0 + pcol + i;
+    for (int i = 0; i < PX; ++i) {
+      int y, x;
+      pos(lane + 32 * i, y, x);
       const bool in = y < a.H && x < a.W;
       const int64_t pix = ((int64_t)p * a.H + min(y, a.H - 1)) * a.W + min(x, a.W - 1);
-      float rv[NC];
+      float rv[NC], pm = 0.f, pr = 0.f;
 #pragma unroll
       for (int j = 0; j < NC; j += 4) {  // the residual, 16 bytes at a time
         float4 r4 = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -231,19 +319,17 @@ __global__ void __launch_bounds__(256) k_conv_simt(ConvParams a) {
         } else if (in) {
           v += rv[j];
         }
-        pm[i] = fmaf(a.wh[co], v, pm[i]);
-        pr[i] = fmaf(a.wh[a.cout_total + co], v, pr[i]);
+        pm = fmaf(a.wh[co], v, pm);
+        pr = fmaf(a.wh[a.cout_total + co], v, pr);
       }
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      s_head[cg][prow * TW + pcol + i][0] = pm[i];
-      s_head[cg][prow * TW + pcol + i][1] = pr[i];
+      s_head[cg][lane + 32 * i][0] = pm;
+      s_head[cg][lane + 32 * i][1] = pr;
     }
     __syncthreads();
-    if (t < TH * TW) {
-      const int yy = y0 + t / TW, xx = x0 + t % TW;
-      if (yy < a.H && xx < a.W && step_of(yy, xx) == a.step) {
+    if (t < G::TH * G::TW) {
+      int yy, xx;
+      pos(t, yy, xx);
+      if (yy < a.H && xx < a.W) {
         float mu = a.bh[0], rho = a.bh[1];
 #pragma unroll
         for (int g = 0; g < 8; ++g) { mu += s_head[g][t][0]; rho += s_head[g][t][1]; }
@@ -273,94 +359,120 @@ __global__ void __launch_bounds__(256) k_conv_simt(ConvParams a) {
   }
 }
 
+// The SIMT producers below: one block per row (plane p, row y), a thread has
+// 4 fixed channels (their 9 taps in registers) and walks the row; per output
+// the bias, then the taps in raster order.
+struct Taps4 {
+  float w[4][9], b[4];
+  __device__ __forceinline__ Taps4(const float *wt, const float *bias, int c) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+#pragma unroll
+      for (int t = 0; t < 9; ++t) w[k][t] = __ldg(wt + (c + k) * 9 + t);
+      b[k] = __ldg(bias + c + k);
+    }
+  }
+};
+__device__ __forceinline__ float4 rq4(const float *v, int rqn) {
+  if (rqn == kRqFloat) return make_float4(v[0], v[1], v[2], v[3]);
+  return make_float4(rq_f(v[0], rqn, 127), rq_f(v[1], rqn, 127), rq_f(v[2], rqn, 127),
+                     rq_f(v[3], rqn, 127));
+}
+
 // ConvLSTM input: X[..., 0:C] = conv3x3(1->C)(up(s_prev)) + be,
 // X[..., C:2C] = up(h_prev) (zero for the first LSTM step).
-__global__ void k_lstm_in(const int32_t *__restrict__ s_prev, const float *__restrict__ h_prev,
-                          int h_cs, int h_co, const float *__restrict__ we,
-                          const float *__restrict__ be, float *__restrict__ X, int P, int H,
-                          int W, int C, int up, int first, int rqn) {
-  const int64_t n = (int64_t)P * H * W * C;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int c = (int)(e % C);
-    const int64_t pix = e / C;
-    const int x = (int)(pix % W);
-    const int y = (int)((pix / W) % H);
-    const int p = (int)(pix / ((int64_t)W * H));
-    const int Hp = H >> up, Wp = W >> up;
-    const int32_t *sp = s_prev + (int64_t)p * Hp * Wp;
-    float v = be[c];
+__global__ void __launch_bounds__(256) k_lstm_in(
+    const int32_t *__restrict__ s_prev, const float *__restrict__ h_prev, int h_cs, int h_co,
+    const float *__restrict__ we, const float *__restrict__ be, float *__restrict__ X, int H,
+    int W, int C, int up, int first, int rqn) {
+  const int y = blockIdx.x % H;
+  const int64_t p = blockIdx.x / H;
+  const int c = 4 * (threadIdx.x % (C / 4)), nx = blockDim.x / (C / 4);
+  const Taps4 k(we, be, c);
+  const int Hp = H >> up, Wp = W >> up;
+  const int32_t *sp = s_prev + p * Hp * Wp;
+  for (int x = threadIdx.x / (C / 4); x < W; x += nx) {
+    float v[4] = {k.b[0], k.b[1], k.b[2], k.b[3]};
 #pragma unroll
     for (int tap = 0; tap < 9; ++tap) {
       const int yy = y + tap / 3 - 1, xx = x + tap % 3 - 1;
       if (yy < 0 || yy >= H || xx < 0 || xx >= W) continue;
-      int32_t sv = sp[(int64_t)(yy >> up) * Wp + (xx >> up)];
+      int32_t sv = __ldg(sp + (int64_t)(yy >> up) * Wp + (xx >> up));
       if (rqn != kRqFloat) sv = min(max(sv, -127), 127);   // integer class input
-      v = fmaf(we[c * 9 + tap], (float)sv, v);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) v[q] = fmaf(k.w[q][tap], (float)sv, v[q]);
     }
-    X[pix * 2 * C + c] = rqn != kRqFloat ? rq_f(v, rqn, 127) : v;
-    float hv = 0.f;
-    if (!first) {
-      const int64_t pp = ((int64_t)p * Hp + (y >> up)) * Wp + (x >> up);
-      hv = h_prev[pp * h_cs + h_co + c];
-    }
-    X[pix * 2 * C + C + c] = hv;
+    float *o = X + ((p * H + y) * W + x) * 2 * C + c;
+    *reinterpret_cast<float4 *>(o) = rq4(v, rqn);
+    float4 h = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (!first)
+      h = *reinterpret_cast<const float4 *>(
+          h_prev + ((p * Hp + (y >> up)) * Wp + (x >> up)) * h_cs + h_co + c);
+    *reinterpret_cast<float4 *>(o + C) = h;
   }
 }
 
 // Masked spatial input of steps 2-4: out[..., 0:C] = conv3x3(1->C)(m_<k s) + b.
-__global__ void k_masked_in(const int32_t *__restrict__ s, const float *__restrict__ wa,
-                            const float *__restrict__ ba, float *__restrict__ out, int out_cs,
-                            int P, int H, int W, int C, int step, int rqn) {
-  const int64_t n = (int64_t)P * H * W * C;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int c = (int)(e % C);
-    const int64_t pix = e / C;
-    const int x = (int)(pix % W);
-    const int y = (int)((pix / W) % H);
-    const int p = (int)(pix / ((int64_t)W * H));
-    const int32_t *sp = s + (int64_t)p * H * W;
-    float v = ba[c];
+__global__ void __launch_bounds__(256) k_masked_in(const int32_t *__restrict__ s,
+                                                   const float *__restrict__ wa,
+                                                   const float *__restrict__ ba,
+                                                   float *__restrict__ out, int out_cs, int H,
+                                                   int W, int C, int step, int rqn) {
+  const int y = blockIdx.x % H;
+  const int64_t p = blockIdx.x / H;
+  // taps of an earlier step, by x mod 4 (the pattern's period)
+  __shared__ uint32_t smask[4];
+  if (threadIdx.x < 4) {
+    uint32_t m = 0;
+    for (int tap = 0; tap < 9; ++tap)
+      if (step_of(y + 2 + tap / 3 - 1, threadIdx.x + 4 + tap % 3 - 1) < step) m |= 1u << tap;
+    smask[threadIdx.x] = m;
+  }
+  const int c = 4 * (threadIdx.x % (C / 4)), nx = blockDim.x / (C / 4);
+  const Taps4 k(wa, ba, c);
+  __syncthreads();
+  const int32_t *sp = s + p * H * W;
+  for (int x = threadIdx.x / (C / 4); x < W; x += nx) {
+    const uint32_t m = smask[x & 3];
+    float v[4] = {k.b[0], k.b[1], k.b[2], k.b[3]};
 #pragma unroll
     for (int tap = 0; tap < 9; ++tap) {
       const int yy = y + tap / 3 - 1, xx = x + tap % 3 - 1;
-      if (yy < 0 || yy >= H || xx < 0 || xx >= W) continue;
-      if (step_of(yy, xx) >= step) continue;
-      int32_t sv = sp[(int64_t)yy * W + xx];
+      if (!((m >> tap) & 1u) || yy < 0 || yy >= H || xx < 0 || xx >= W) continue;
+      int32_t sv = __ldg(sp + (int64_t)yy * W + xx);
       if (rqn != kRqFloat) sv = min(max(sv, -127), 127);   // integer class input
-      v = fmaf(wa[c * 9 + tap], (float)sv, v);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) v[q] = fmaf(k.w[q][tap], (float)sv, v[q]);
     }
-    out[pix * out_cs + c] = rqn != kRqFloat ? rq_f(v, rqn, 127) : v;
+    *reinterpret_cast<float4 *>(out + ((p * H + y) * W + x) * out_cs + c) = rq4(v, rqn);
   }
 }
 
 // Depthwise 3x3 (zero padding): out = dw(in) + b, NHWC with C channels.
-__global__ void k_dw3x3(const float *__restrict__ in, const float *__restrict__ w,
-                        const float *__restrict__ b, float *__restrict__ out, int P, int H,
-                        int W, int C, int rqn) {
-  const int64_t n = (int64_t)P * H * W * C;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int c = (int)(e % C);
-    const int64_t pix = e / C;
-    const int x = (int)(pix % W);
-    const int y = (int)((pix / W) % H);
-    const int64_t pbase = pix - ((int64_t)y * W + x);
-    float v = b[c];
+__global__ void __launch_bounds__(256) k_dw3x3(const float *__restrict__ in,
+                                               const float *__restrict__ w,
+                                               const float *__restrict__ b,
+                                               float *__restrict__ out, int H, int W, int C,
+                                               int rqn) {
+  const int y = blockIdx.x % H;
+  const int64_t p = blockIdx.x / H;
+  const int c = 4 * (threadIdx.x % (C / 4)), nx = blockDim.x / (C / 4);
+  const Taps4 k(w, b, c);
+  const float *ip = in + p * H * W * C + c;
+  for (int x = threadIdx.x / (C / 4); x < W; x += nx) {
+    float v[4] = {k.b[0], k.b[1], k.b[2], k.b[3]};
 #pragma unroll
     for (int tap = 0; tap < 9; ++tap) {
       const int yy = y + tap / 3 - 1, xx = x + tap % 3 - 1;
       if (yy < 0 || yy >= H || xx < 0 || xx >= W) continue;
-      v = fmaf(w[c * 9 + tap], in[(pbase + (int64_t)yy * W + xx) * C + c], v);
+      const float4 f = __ldg(reinterpret_cast<const float4 *>(ip + ((int64_t)yy * W + xx) * C));
+      v[0] = fmaf(k.w[0][tap], f.x, v[0]);
+      v[1] = fmaf(k.w[1][tap], f.y, v[1]);
+      v[2] = fmaf(k.w[2][tap], f.z, v[2]);
+      v[3] = fmaf(k.w[3][tap], f.w, v[3]);
     }
-    out[pix * C + c] = rqn != kRqFloat ? rq_f(v, rqn, 127) : v;
+    *reinterpret_cast<float4 *>(out + ((p * H + y) * W + x) * C + c) = rq4(v, rqn);
   }
-}
-
-static int grid_for(int64_t n) {
-  int64_t g = (n + 255) / 256;
-  return (int)(g > 152 * 64 ? 152 * 64 : (g < 1 ? 1 : g));
 }
 
 bool &launch_failed() {
@@ -368,22 +480,53 @@ bool &launch_failed() {
   return f;
 }
 
+template <int KS, int WG, int NC, int PX, int EPI>
+static void launch_simt_cfg(const ConvParams &a, cudaStream_t st) {
+  using G = SimtCfg<KS, WG, NC, PX, EPI>;
+  static std::atomic<uint64_t> attr{0};
+  once_per_device(attr, [] {
+    cudaFuncSetAttribute(k_conv_simt<KS, WG, NC, PX, EPI>,
+                         cudaFuncAttributeMaxDynamicSharedMemorySize, G::kSmem);
+  });
+  const int npos = G::kStep ? std::max(row_count(a.W, step_phase(a.step, 0)),
+                                       row_count(a.W, step_phase(a.step, 1)))
+                            : a.W;
+  const int tiles = ((a.H + G::TH - 1) / G::TH) * ((npos + G::TW - 1) / G::TW);
+  if (tiles == 0) return;   // a head of a step without positions
+  k_conv_simt<KS, WG, NC, PX, EPI>
+      <<<dim3(tiles, a.cout_total / G::CO, a.P), 32 * WG, G::kSmem, st>>>(a);
+}
+
 void launch_conv_simt(int ks, const ConvParams &a, int epi, cudaStream_t st) {
-  const int tiles = ((a.H + 7) / 8) * ((a.W + 15) / 16);
-  int co_t = a.cout_total >= 64 ? 64 : 32;
-  if (epi == EPI_HEAD) co_t = a.cout_total;
-  dim3 grid(tiles, (a.cout_total + co_t - 1) / co_t, a.P);
-#define PW_CONV_CASE(KS_, CO_, EPI_)                                         \
-  if (ks == KS_ && co_t == CO_ && epi == EPI_) {                             \
-    k_conv_simt<KS_, CO_, EPI_><<<grid, 256, 0, st>>>(a);                    \
-    return;                                                                  \
+  // Large blocks (128 positions x 32 or 64 channels, 8 warps) where they give
+  // every SM at least two; else small ones, 64 positions x 8 channels in 2
+  // warps (the shared-memory port of an SM then serves few warps, and a tiny
+  // plane spreads over the SMs). The head has all channels in a block: 128 or
+  // 32 positions.
+  const int64_t px = (int64_t)((a.H + 7) / 8) * ((a.W + 15) / 16) * a.P;
+  const int co = a.cout_total;
+  const bool c64 = co >= 64;
+  const bool large = epi == EPI_HEAD ? px / 4 >= 2 * sm_count()
+                                     : px * (co / (c64 ? 64 : 32)) >= 2 * sm_count();
+  const bool fits = co % 32 == 0 && (!c64 || co % 64 == 0) && a.cin % 32 == 0;
+#define PW_CONV_CASE(KS_, EPI_)                                                      \
+  if (fits && ks == KS_ && epi == EPI_) {                                            \
+    if (!large) launch_simt_cfg<KS_, 2, 4, 2, EPI_>(a, st);                          \
+    else if (c64) launch_simt_cfg<KS_, 8, 8, 4, EPI_>(a, st);                        \
+    else launch_simt_cfg<KS_, 8, 4, 4, EPI_>(a, st);                                 \
+    return;                                                                          \
   }
-  PW_CONV_CASE(1, 32, EPI_STORE) PW_CONV_CASE(1, 64, EPI_STORE)
-  PW_CONV_CASE(3, 32, EPI_STORE) PW_CONV_CASE(3, 64, EPI_STORE)
-  PW_CONV_CASE(3, 32, EPI_LSTM) PW_CONV_CASE(3, 64, EPI_LSTM)
-  PW_CONV_CASE(1, 32, EPI_HEAD) PW_CONV_CASE(1, 64, EPI_HEAD) PW_CONV_CASE(1, 128, EPI_HEAD)
-  PW_CONV_CASE(3, 32, EPI_HEAD) PW_CONV_CASE(3, 64, EPI_HEAD) PW_CONV_CASE(3, 128, EPI_HEAD)
+#define PW_HEAD_CASE(KS_, C_)                                                        \
+  if (fits && ks == KS_ && epi == EPI_HEAD && co == C_) {                            \
+    if (!large) launch_simt_cfg<KS_, 8, C_ / 8, 1, EPI_HEAD>(a, st);                 \
+    else launch_simt_cfg<KS_, 8, C_ / 8, 4, EPI_HEAD>(a, st);                        \
+    return;                                                                          \
+  }
+  PW_CONV_CASE(1, EPI_STORE) PW_CONV_CASE(3, EPI_STORE) PW_CONV_CASE(3, EPI_LSTM)
+  PW_HEAD_CASE(1, 32) PW_HEAD_CASE(1, 64) PW_HEAD_CASE(1, 128)
+  PW_HEAD_CASE(3, 32) PW_HEAD_CASE(3, 64) PW_HEAD_CASE(3, 128)
 #undef PW_CONV_CASE
+#undef PW_HEAD_CASE
   set_last_error("no convolution kernel for this shape");
   launch_failed() = true;
 }
@@ -391,20 +534,17 @@ void launch_conv_simt(int ks, const ConvParams &a, int epi, cudaStream_t st) {
 void launch_lstm_in(const int32_t *s_prev, const float *h_prev, int h_cs, int h_co,
                     const float *we, const float *be, float *X, int P, int H, int W, int C,
                     int up, int first, cudaStream_t st, int rqn) {
-  int64_t n = (int64_t)P * H * W * C;
-  k_lstm_in<<<grid_for(n), 256, 0, st>>>(s_prev, h_prev, h_cs, h_co, we, be, X, P, H, W, C,
-                                          up, first, rqn);
+  k_lstm_in<<<P * H, 256, 0, st>>>(s_prev, h_prev, h_cs, h_co, we, be, X, H, W, C, up, first,
+                                   rqn);
 }
 void launch_masked_in(const int32_t *s, const float *wa, const float *ba, float *out,
                       int out_cs, int P, int H, int W, int C, int step, cudaStream_t st,
                       int rqn) {
-  int64_t n = (int64_t)P * H * W * C;
-  k_masked_in<<<grid_for(n), 256, 0, st>>>(s, wa, ba, out, out_cs, P, H, W, C, step, rqn);
+  k_masked_in<<<P * H, 256, 0, st>>>(s, wa, ba, out, out_cs, H, W, C, step, rqn);
 }
 void launch_dw3x3(const float *in, const float *w, const float *b, float *out, int P, int H,
                   int W, int C, cudaStream_t st, int rqn) {
-  int64_t n = (int64_t)P * H * W * C;
-  k_dw3x3<<<grid_for(n), 256, 0, st>>>(in, w, b, out, P, H, W, C, rqn);
+  k_dw3x3<<<P * H, 256, 0, st>>>(in, w, b, out, H, W, C, rqn);
 }
 
 }  // namespace pw
