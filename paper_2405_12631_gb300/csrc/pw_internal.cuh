@@ -134,9 +134,11 @@ __host__ __device__ __forceinline__ int step_phase(int k, int row_odd) {
   return ((row_odd ? odd : even) >> (2 * k)) & 3;
 }
 __host__ __device__ __forceinline__ int step_of(int y, int x) {
-  const int ev[4] = {0, 2, 1, 3};   // x % 4 -> step (even rows)
-  const int od[4] = {1, 3, 0, 2};   // x % 4 -> step (odd rows)
-  return (y & 1) ? od[x & 3] : ev[x & 3];
+  // x % 4 -> step, two bits each (as arrays they would be indexed in local
+  // memory)
+  const int even = (0) | (2 << 2) | (1 << 4) | (3 << 6);
+  const int odd = (1) | (3 << 2) | (0 << 4) | (2 << 6);
+  return (((y & 1) ? odd : even) >> (2 * (x & 3))) & 3;
 }
 __host__ __device__ __forceinline__ int row_count(int w, int a) {
   return w > a ? (w - a + 3) >> 2 : 0;
