@@ -845,6 +845,14 @@ __global__ void __launch_bounds__(conv_threads(KS, EPI, NCTA), 1) k_conv_tc(cons
         for (int g = 0; g < NH / 32; ++g)
           store_bf16x8(a.out + (((int64_t)p * G + a.out_goff + (ch0 >> 3) + g) * hw + pix) * 8,
                        hv + 8 * g);
+        if (!F8 && a.outc && step_of(y, x) == 0) {
+          // the step-1 positions' h once more, dense, for that step's net
+          const int64_t qn = step_index(a.W, 0, y, x);
+#pragma unroll
+          for (int g = 0; g < NH / 32; ++g)
+            store_bf16x8(a.outc + (((int64_t)p * G + (ch0 >> 3) + g) * a.outc_n + qn) * 8,
+                         hv + 8 * g);
+        }
         if (a.out8) {
           // 8 channels (half of a 16-byte group) at a time
 #pragma unroll
@@ -982,46 +990,88 @@ __global__ void __launch_bounds__(256) k_copy_up16(const uint4 *__restrict__ src
 
 // Compact step tail input: for the q-th position (y, x) of step `step`,
 // Vc[q] = dw3x3(U)(y, x) + b and Zc[q] = Z(y, x) (C channels each, blocked
-// layout; q indexes the compact plane of hc x wc positions).
-__global__ void __launch_bounds__(256) k_dw3x3_compact(
+// layout; q indexes the compact plane of hc x wc positions: xc < ne lies on
+// row 2 yc, the rest on row 2 yc + 1). Without Z, Zc is there already.
+// A block takes one channel group of one plane and kDwThreads * per
+// consecutive positions, so that a thread reads the group's 72 weights once
+// and keeps them in registers; one weight read for each product from shared
+// memory was the time of the small planes (one 2047 x 1365 scan: 22.4 us a
+// launch, 15.7 with the weights in registers). A large plane is bound by
+// memory: all of U, and of Z every 64 bytes for the 16 of one position, which
+// is 40 % of the traffic (5.7 TB/s under a profiler). The BF16 gates therefore write
+// their step-1 positions densely beside h: this pass in a GOP of 8 frames of
+// 1920 x 1080 4.3-4.6 -> 3.1 ms, the scan's 13.1 us a launch, for 0.1-0.3 ms
+// of the GOP's gates. The FP8 gates are bound by their epilogue (a batch of 24
+// images of 768 x 512: gates 4.37 -> 4.76 ms for 1.63 -> 1.28 here), so there
+// the positions are gathered.
+constexpr int kDwThreads = 128;
+__global__ void __launch_bounds__(kDwThreads, 4) k_dw3x3_compact(
     const __nv_bfloat16 *__restrict__ U, const __nv_bfloat16 *__restrict__ Z,
     const float *__restrict__ w, const float *__restrict__ b, __nv_bfloat16 *__restrict__ Vc,
-    __nv_bfloat16 *__restrict__ Zc, int P, int H, int W, int C, int step, int n, int64_t chw) {
-  // one block per compact row (plane p, row pair yc); item = group-major
-  // (g, xc); xc < n_even lies on row 2 yc, the rest on row 2 yc + 1
-  __shared__ float sw[9 * 128], sb[128];
-  for (int i = threadIdx.x; i < 9 * C; i += blockDim.x) sw[i] = w[i];
-  for (int i = threadIdx.x; i < C; i += blockDim.x) sb[i] = b[i];
-  __syncthreads();
-  const int G = C / 8;
+    __nv_bfloat16 *__restrict__ Zc, int H, int W, int G, int step, int per, int nblk) {
+  const int64_t pg = blockIdx.x / nblk;            // p * G + g
+  const int g = (int)(pg % G);
   const int hc = (H + 1) >> 1;
-  const int yc = blockIdx.x % hc;
-  const int64_t p = blockIdx.x / hc;
   const int ae = step_phase(step, 0), ao = step_phase(step, 1);
   const int ne = row_count(W, ae), wc = ne + row_count(W, ao);
+  const int chw = hc * wc;
+  int q = (blockIdx.x % nblk) * (kDwThreads * per) + threadIdx.x;
+  if (q >= chw) return;
+  float wk[8][9], bk[8];
+  {
+    const float4 *w4 = reinterpret_cast<const float4 *>(w + 72 * g);
+#pragma unroll
+    for (int i = 0; i < 18; ++i) {
+      const float4 t = __ldg(w4 + i);
+      const float e[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+      for (int k = 0; k < 4; ++k) wk[(4 * i + k) / 9][(4 * i + k) % 9] = e[k];
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) bk[k] = __ldg(b + 8 * g + k);
+  }
   const int64_t hw = (int64_t)H * W;
-  for (int it = threadIdx.x; it < G * wc; it += blockDim.x) {
-    const int g = it / wc, xc = it - g * wc;
+  const uint4 *u0 = reinterpret_cast<const uint4 *>(U) + pg * hw;
+  const uint4 *z0 = reinterpret_cast<const uint4 *>(Z) + pg * hw;
+  uint4 *zc = reinterpret_cast<uint4 *>(Zc) + pg * chw;
+  int yc = q / wc, xc = q - yc * wc;
+  const int dy = kDwThreads / wc, dx = kDwThreads - dy * wc;
+#pragma unroll 1
+  for (int i = 0; i < per && q < chw; ++i, q += kDwThreads) {
     const int y = xc < ne ? 2 * yc : 2 * yc + 1;
     const int x = xc < ne ? ae + 4 * xc : ao + 4 * (xc - ne);
-    if (y >= H) continue;  // odd height: the last pair has no odd row
-    const int64_t pg = p * G + g;
-    float v[8];
+    if (y < H) {  // odd height: the last pair has no odd row
+      const uint4 *c = u0 + (int64_t)y * W + x;
+      const uint4 zv = Z ? z0[(int64_t)y * W + x] : make_uint4(0u, 0u, 0u, 0u);
+      float v[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) v[k] = sb[8 * g + k];
+      for (int k = 0; k < 8; ++k) v[k] = bk[k];
+      auto tap = [&](int t, const uint4 &r) {
+        const uint32_t e[4] = {r.x, r.y, r.z, r.w};
 #pragma unroll
-    for (int tap = 0; tap < 9; ++tap) {
-      const int yy = y + tap / 3 - 1, xx = x + tap % 3 - 1;
-      if (yy < 0 || yy >= H || xx < 0 || xx >= W) continue;
-      float u[8];
-      load_bf16x8(U + (pg * hw + (int64_t)yy * W + xx) * 8, u);
+        for (int k = 0; k < 8; ++k)
+          v[k] = fmaf(wk[k][t], __uint_as_float(k & 1 ? e[k >> 1] & 0xffff0000u : e[k >> 1] << 16),
+                      v[k]);
+      };
+      if (y > 0 && y + 1 < H && x > 0 && x + 1 < W) {
+        uint4 r[9];
 #pragma unroll
-      for (int k = 0; k < 8; ++k) v[k] = fmaf(sw[(8 * g + k) * 9 + tap], u[k], v[k]);
+        for (int t = 0; t < 9; ++t) r[t] = c[(int64_t)(t / 3 - 1) * W + t % 3 - 1];
+#pragma unroll
+        for (int t = 0; t < 9; ++t) tap(t, r[t]);
+      } else {
+#pragma unroll
+        for (int t = 0; t < 9; ++t) {
+          const int yy = y + t / 3 - 1, xx = x + t % 3 - 1;
+          if (yy >= 0 && yy < H && xx >= 0 && xx < W)
+            tap(t, c[(int64_t)(t / 3 - 1) * W + t % 3 - 1]);
+        }
+      }
+      store_bf16x8(Vc + (pg * chw + q) * 8, v);
+      if (Z) zc[q] = zv;
     }
-    const int64_t q = (int64_t)yc * wc + xc;
-    store_bf16x8(Vc + (pg * chw + q) * 8, v);
-    *reinterpret_cast<uint4 *>(Zc + (pg * chw + q) * 8) =
-        *reinterpret_cast<const uint4 *>(Z + (pg * hw + (int64_t)y * W + x) * 8);
+    yc += dy; xc += dx;
+    if (xc >= wc) { xc -= wc; ++yc; }
   }
 }
 
@@ -1037,7 +1087,7 @@ __global__ void __launch_bounds__(256) k_dw3x3_compact(
 // of 256 x 384 take 54 us (4.7 TB/s). With nine loads, conversions and selects
 // a position it was bound by its instructions: the 39 launches of a batch of
 // 24 images of 768 x 512 took 1.02 ms, now 0.67; those of one image 5.9 us
-// each, now 3.3; of one 1754 x 1240 scan 10.3 us, now 5.3.
+// each, now 3.3; of one 2047 x 1365 scan 10.3 us, now 5.3.
 __device__ __forceinline__ uint32_t bf16_pair(float lo, float hi) {
   const __nv_bfloat162 t = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t *>(&t);
@@ -1991,6 +2041,7 @@ int tc_run_lstm(pw_ctx *ctx, Model &m, const Geometry &g, Workspace &ws, int sb,
   a.c_new = reinterpret_cast<__nv_bfloat16 *>(ws.Cst[cur ^ 1]);
   a.up = up; a.first = first; a.C = C;
   if (f8) { a.out8 = t.L8[sb & 1]; a.out8_G16 = G16; a.out8_scale = m.tc->h_scale; }
+  else { a.outc = t.Zc; a.outc_n = (int)compact_elems(h, w); }
   // MMA work: the 16-channel v block and the C h channels, 9 taps, 4C outputs
   ProfScope ps(ctx, KC_LSTM_GATES, 2.0 * pix * 9 * (16 + C) * 4 * C,
                pix * (32.0 + (f8 ? 1.0 : 2.0) * C + 2.0 * C + 4.0 * C + (f8 ? C : 0)));
@@ -2065,8 +2116,15 @@ int tc_run_step(pw_ctx *ctx, Model &m, const Geometry &g, Workspace &ws, int sb,
     };
     {
       ProfScope ps(ctx, KC_SMALL_CTX, 2.0 * cpix * 9 * C, cpix * 2.0 * C * 4);
-      k_dw3x3_compact<<<P * hc, 256, 0, st>>>(
-          t.U, l, n.wdw, n.bdw, t.Vc, t.Zc, P, h, w, C, 0, n0, chw);  // Zc <- l gathered
+      // the BF16 gates leave l's step-1 positions in Zc (LL has no gates)
+      const bool zc_done = !ll && ctx->precision != PW_PREC_FP8;
+      // a block's positions: four passes over the weights' one load where that
+      // still gives every SM its four blocks twice
+      const int one = (int)((chw + kDwThreads - 1) / kDwThreads);
+      const int per = (int64_t)P * G * one >= 4 * 8 * 152 ? 4 : 1;
+      const int nblk = (one + per - 1) / per;
+      k_dw3x3_compact<<<P * G * nblk, kDwThreads, 0, st>>>(
+          t.U, zc_done ? nullptr : l, n.wdw, n.bdw, t.Vc, t.Zc, h, w, G, 0, per, nblk);
       ctx->launches += 1;
     }
     // the block input z = Win l + bin on the step-1 positions (compact, in Z)
