@@ -683,10 +683,32 @@ __global__ void __launch_bounds__(conv_threads(KS, EPI, NCTA), 1) k_conv_tc(cons
     uint4 cpq[NCP];      // operands of the next tile to process
     uint4 presq[NRES];
     // only the epilogues that read such operands pay for the lookahead (the
-    // z conv never has a residual, conv 1 and most plain stores neither)
-    constexpr bool PREF = EPI == TE_LSTM || HEADK || EPI == TE_STORE;
+    // z conv never has a residual, conv 1 and most plain stores neither; a
+    // plain store of FP8 operands takes none)
+    constexpr bool PREF = EPI == TE_LSTM || HEADK || (EPI == TE_STORE && !F8);
     const bool has_ops = PREF && (EPI != TE_STORE || a.res != nullptr);
     if (has_ops && cta < a.tiles) load_ops(ti, cpq, presq);
+    // A warp's columns are the same in every tile: the 3x3 plain stores' 16
+    // keep their bias, and the FP8 operands' scale, in registers instead of
+    // reading them again for every tile (BF16 conv 1 of a GOP of 8 frames of
+    // 1920 x 1080: 12.54 -> 12.12 ms; FP8 conv 1 of a batch of 24 images of
+    // 768 x 512 4.21 -> 3.70 ms, together with the residual operands that it
+    // never has taken out: with them the constants spilled and gained
+    // nothing). The 1x1 kernels wait for memory, and tighter registers cost
+    // them 2-3 %; of the FP8 gates' 64 constants the bias alone gained nothing.
+    constexpr bool KREG = STORE && KS == 3 && NH <= 16;
+    constexpr bool KSC = KREG && F8;
+    const bool scale_acc = F8 || fold8;
+    uint64_t kbia[KREG ? NH / 2 : 1], ksc[KSC ? NH / 2 : 1];
+    if constexpr (KREG) {
+      const uint64_t *b2 = reinterpret_cast<const uint64_t *>(s_bias + col0);
+      const uint64_t *s2 = reinterpret_cast<const uint64_t *>(s_wsc + col0);
+#pragma unroll
+      for (int j = 0; j < NH / 2; ++j) {
+        kbia[j] = b2[j];
+        if (KSC) ksc[KSC ? j : 0] = s2[j];
+      }
+    }
     for (int t = cta; t < a.tiles;
          t += nctas, ti.next(a.step_dx, a.step_dy, a.step_dp, a.tiles_x, a.tiles_y)) {
       const int p = ti.p;
@@ -731,15 +753,17 @@ __global__ void __launch_bounds__(conv_threads(KS, EPI, NCTA), 1) k_conv_tc(cons
         // column pairs in packed FP32 (per element the same fmaf / add)
         const uint64_t *wsc2 = reinterpret_cast<const uint64_t *>(s_wsc + col0);
         const uint64_t *bia2 = reinterpret_cast<const uint64_t *>(s_bias + col0);
-        if (F8 || fold8) {
+        if (scale_acc) {
 #pragma unroll
           for (int j = 0; j < NH / 2; ++j)
-            f2unpack(fma2(f2pack(v[2 * j], v[2 * j + 1]), wsc2[j], bia2[j]), v[2 * j],
-                     v[2 * j + 1]);
+            f2unpack(fma2(f2pack(v[2 * j], v[2 * j + 1]), KSC ? ksc[KSC ? j : 0] : wsc2[j],
+                          KREG ? kbia[KREG ? j : 0] : bia2[j]),
+                     v[2 * j], v[2 * j + 1]);
         } else {
 #pragma unroll
           for (int j = 0; j < NH / 2; ++j)
-            f2unpack(add2(f2pack(v[2 * j], v[2 * j + 1]), bia2[j]), v[2 * j], v[2 * j + 1]);
+            f2unpack(add2(f2pack(v[2 * j], v[2 * j + 1]), KREG ? kbia[KREG ? j : 0] : bia2[j]),
+                     v[2 * j], v[2 * j + 1]);
         }
       } else if (F8) {
 #pragma unroll
@@ -781,7 +805,7 @@ __global__ void __launch_bounds__(conv_threads(KS, EPI, NCTA), 1) k_conv_tc(cons
       if (STORE) {
 #pragma unroll
         for (int g = 0; g < NH / 8; ++g) {
-          if (a.res) {
+          if (PREF && a.res) {
             float rv[8];
             load_bf16x8(reinterpret_cast<const __nv_bfloat16 *>(&pres[g]), rv);
 #pragma unroll
@@ -1452,6 +1476,10 @@ static int conv_tc(pw_ctx *ctx, const TcWeights::Conv &cv, const void *in, int i
       a.hstage_bytes = 0;
       a.nkb += 1;
     }
+  }
+  if (a.epi == TE_STORE && cv.f8 && a.res) {
+    set_last_error("no residual in a plain store of FP8 operands");
+    return PW_EUNSUPPORTED;
   }
   if ((a.epi == TE_LSTM || a.epi == TE_STOREV) != (cv.wv != nullptr)) {
     set_last_error("tensor-core conv: v block and epilogue do not match");
