@@ -293,7 +293,7 @@ int pw_rans_encode(pw_ctx *ctx, int nchunks, const uint32_t *count,
  * PW_ECORRUPT (a corrupt or truncated chunk, and also a chunk whose offset +
  * nbytes exceeds payload_bytes or whose lane count is not 1..32: the checks
  * run on the device, where pw_rans_decode reports those two as PW_EINVAL),
- * PW_ETIMEOUT (the decoder's bounded wait for its table copy expired),
+ * PW_ETIMEOUT (reserved for a bounded wait; the decoder waits on none),
  * PW_EUNSUPPORTED, PW_ECUDA. */
 int pw_rans_decode_noalloc(void *cuda_stream, const uint8_t *payload, size_t payload_bytes,
                            int nchunks, const uint32_t *offset, const uint32_t *nbytes,

@@ -152,7 +152,7 @@ extern "C" int pw_rans_decode_noalloc(void *cuda_stream, const uint8_t *payload,
     return PW_EINVAL;
   }
   if (h & kStTimeout) {
-    set_last_error("the decoder's bounded wait for its table copy expired");
+    set_last_error("a kernel's bounded wait expired");
     return PW_ETIMEOUT;
   }
   if (h) {
