@@ -599,6 +599,7 @@ __global__ void __launch_bounds__(768) k_rans_decode(
                   if (!tail) {
                     const int c = min(__ffs(~bits) - 1, n);
                     kcnt += c;
+                    if (kcnt > kMaxEscBits) bad = true;   // also when the zero follows
                     left -= c;
                     if (left > 0) {
                       tail = true;
@@ -613,7 +614,6 @@ __global__ void __launch_bounds__(768) k_rans_decode(
                     kcnt -= q;
                     left -= q;
                   }
-                  if (!tail && kcnt > kMaxEscBits) bad = true;
                   x = ((x >> (14 + n - left)) << 14) | (x & 0x3FFFu);
                   nd = left == 0;
                   if (pass == 0) e = n - 1;

@@ -1,0 +1,154 @@
+"""rANS decoder on hand-made chunks: escape prefixes up to the limit give
+their values, longer ones are reported. The oracle's coder writes the chunks
+from explicit coding operations, so that a prefix may have any length."""
+import numpy as np
+import pytest
+
+import synthetic as S
+from oracle import codec as K
+from oracle import entropy as E
+from oracle import rans as R
+from tests._lib import ensure_built
+from tests.test_zz_no_alloc import _noalloc
+
+pytestmark = pytest.mark.gpu
+ensure_built()
+
+KMAX = 30                                   # longest escape prefix of the format
+
+
+@pytest.fixture(scope="module")
+def pw():
+    import paper_2405_12631_gb300 as m
+    return m
+
+
+@pytest.fixture(scope="module")
+def codec(pw):
+    c = pw.Codec(0, "fp32")
+    yield c
+    c.close()
+
+
+@pytest.fixture(scope="module")
+def bank():
+    return E.cdf_bank().astype(np.int64)
+
+
+def _esc_ops(cdf, right, k, low):
+    """An escape of k ones, a zero and the k bits of low; and its residual."""
+    s = R.ESC_R if right else R.ESC_L
+    bits = [1] * k + [0] + [(low >> (k - 1 - i)) & 1 for i in range(k)]
+    ops = [(int(cdf[s]), int(cdf[s + 1]) - int(cdf[s]))] + [(b * R.HALF, R.HALF) for b in bits]
+    e = (1 << k) + low - 1
+    return ops, (e if right else -e) + (R.T + 1 if right else -R.T - 1)
+
+
+def _chunk(rng, bank, n, nl, escapes):
+    """n symbols on nl lanes, `escapes` {symbol: prefix length} among small
+    residuals: (payload, packed indices, values)."""
+    tid = rng.integers(0, 2048, n)
+    tid = (tid & ~127) | np.clip(tid & 127, 0, 80)
+    ctr = rng.integers(-30, 30, n)
+    ops, vals = [], []
+    for p in range(n):
+        if p in escapes:
+            k = escapes[p]
+            low = int(rng.integers(0, 1 << k)) if k < KMAX else int(rng.integers(0, (1 << k) - 4096))
+            o, r = _esc_ops(bank[tid[p]], bool(rng.integers(2)), k, low)
+        else:
+            r = int(rng.integers(-3, 4))
+            o = R.symbol_ops(r, bank[tid[p]])
+        ops.append(o)
+        vals.append(int(ctr[p]) + r)
+    st, words = R.encode_chunk(ops, nl)
+    t = 16 * ctr + (tid // 128 - 8)
+    idx = (((t + (1 << 23)) << 7) | (tid % 128)).astype(np.uint32)
+    return R.pack_chunk(st, words), idx, vals
+
+
+def _both(pw, codec, buf, n, nl, idx, nbytes=None):
+    """(status, values) of the regular and the allocation-free decoder."""
+    u32 = lambda v: np.asarray([v], dtype=np.uint32)
+    a = (buf, u32(0), u32(len(buf) if nbytes is None else nbytes), u32(n), u32(nl), idx)
+    try:
+        reg = pw.PW_OK, codec.rans_decode(*a)
+    except pw.PwError as e:
+        reg = e.code, None
+    rc, got = _noalloc(pw, *a)
+    assert rc == reg[0], (rc, reg[0])
+    return rc, got if reg[1] is None else reg[1]
+
+
+@pytest.mark.parametrize("nl", [1, 5, 32])
+@pytest.mark.parametrize("k", [30, 31, 32, 35, 45])
+def test_escape_prefix_limit(pw, codec, bank, nl, k):
+    """The state's fill when the escape starts decides where its passes of up
+    to 16 bits end: 48 chunks with other symbols before it."""
+    rng = np.random.default_rng(100 * nl + k)
+    for _ in range(48):
+        n = int(rng.integers(1, 3 * nl + 2))
+        buf, idx, vals = _chunk(rng, bank, n, nl, {int(rng.integers(0, n)): k})
+        rc, got = _both(pw, codec, buf, n, nl, idx)
+        if k <= KMAX:
+            assert rc == pw.PW_OK and got.tolist() == vals
+        else:
+            assert rc == pw.PW_ECORRUPT, "an over-long prefix was accepted"
+
+
+@pytest.mark.parametrize("nl", [1, 3, 32])
+def test_every_prefix_length(pw, codec, bank, nl):
+    """Prefixes of 0 to 30 at every state, on neighbouring lanes and alone."""
+    rng = np.random.default_rng(nl)
+    n = 40 * 31
+    esc = {p: int(k) for p, k in zip(rng.permutation(n)[:31 * 16], np.tile(np.arange(31), 16))}
+    buf, idx, vals = _chunk(rng, bank, n, nl, esc)
+    rc, got = _both(pw, codec, buf, n, nl, idx)
+    assert rc == pw.PW_OK and got.tolist() == vals
+
+
+@pytest.mark.parametrize("k", [30, 31, 33, 40])
+def test_escape_prefix_limit_ragged(pw, k, monkeypatch):
+    """The last chunk of a stream, on which no other depends, in a ragged
+    batch and alone."""
+    cfg = S.ModelConfig(levels=4, C=32, ll_mode=0)
+    blob = S.pack_blob(cfg, S.random_model(cfg, 1))
+    rng = np.random.default_rng(k)
+    img = S.gray_sinusoids(16, 32, seed=1)
+    encode, tables_of = R.encode_chunk, K.coding_tables
+    tables, seen, last = [None], [0], [0]
+
+    def keep_tables(*args):
+        ctr, tables[0] = tables_of(*args)
+        return ctr, tables[0]
+
+    def escape_in_last(ops, nl):
+        seen[0] += 1
+        if seen[0] == last[0]:
+            p = int(rng.integers(0, len(ops)))
+            ops = list(ops)
+            ops[p], _ = _esc_ops(tables[0][p], True, k, 5)
+        return encode(ops, nl)
+
+    monkeypatch.setattr(K, "coding_tables", keep_tables)
+    monkeypatch.setattr(R, "encode_chunk", escape_in_last)
+    streams = []
+    for _ in range(13):   # the first one as it is
+        seen[0] = 0
+        streams.append(K.encode_image(blob, img, q=8.0, integer=True))
+        last[0] = seen[0]
+    codec = pw.Codec(0, "int8")
+    model = codec.load_model(blob)
+    other = codec.encode_image(model, S.gray_sinusoids(33, 20, seed=2), q=8.0)
+    codec.decode_ragged(model, [other, streams[0]])
+    for bs in streams[1:]:
+        for call in (lambda: codec.decode_ragged(model, [other, bs]),
+                     lambda: codec.decode_symbols(model, bs)):
+            if k <= KMAX:
+                call()
+            else:
+                with pytest.raises(pw.PwError) as e:
+                    call()
+                assert e.value.code == pw.PW_ECORRUPT
+    model.close()
+    codec.close()
