@@ -163,6 +163,10 @@ __device__ __forceinline__ void trio_sync(int id) {
 //    index (for the output) is counted off the chain.
 //  * Lanes without a symbol in a round get a dummy row whose only symbol
 //    fills the interval (the state stays), so the round has no predicates.
+//    Such a lane reads no word as long as its state is at least 2^16, which
+//    every state of an encoder is and stays. A chunk with an initial state
+//    below that is decoded round by round, where only lanes with a symbol
+//    may read.
 //  * Renormalisation: lane l holds word ptr + l of the stream; a lane's word
 //    is one shuffle by its rank among the lanes that need one. Words come
 //    from a ring in shared memory, refilled 64 at a time from a register
@@ -445,6 +449,8 @@ __global__ void __launch_bounds__(768) k_rans_decode(
   const uint32_t nwords = (ch.nbytes - 4u * nl) >> 1;
   const uint8_t *wp = ch.data + 4 * nl;
   uint32_t x = ld_state(ch.data, lane, nl);
+  // (a round and its word leave a state below 2^16 only if it was there)
+  const bool low = __any_sync(0xffffffffu, x < kRansL);
   uint16_t *ring = reinterpret_cast<uint16_t *>(sm + pbase + kRowBufBytes + kResBytes);
   // words k, k + 1 (k = base + 2 lane) into the ring
   auto put = [&](uint32_t k, uint32_t v) {
@@ -538,7 +544,7 @@ __global__ void __launch_bounds__(768) k_rans_decode(
         const uint32_t x0 = x;
         const uint32_t p0 = ptr + took;
         const uint32_t rsg = rs0 + ((b & 1) * kRound + g) * 128u;
-        bool esc = false;
+        bool esc = low;
 #pragma unroll
         for (int u = 0; u < kGroup; ++u) {
           const uint32_t rw = row;
@@ -574,8 +580,12 @@ __global__ void __launch_bounds__(768) k_rans_decode(
               uint32_t m;
               int r;
               round(rw, ldrow(rw, 256u), ldrow(rw, 272u), m, r, [] {});
+              // lanes with a symbol in this round
+              const int nsym = min(nl, max(0, count - (int)it * nl));
+              m &= (uint32_t)((1ull << nsym) - 1);
               while (ptr - wb >= 64u) refill();
-              if (x < kRansL) x = (x << 16) | ring[(ptr & (kRing - 1)) + __popc(m & lt)];
+              if ((m >> lane) & 1u)
+                x = (x << 16) | ring[(ptr & (kRing - 1)) + __popc(m & lt)];
               ptr += __popc(m);
               // Escapes: ones up to a zero, then as many bits, one bypass bit
               // a round, the lanes whose state fell below 2^16 taking a word

@@ -152,3 +152,46 @@ def test_escape_prefix_limit_ragged(pw, k, monkeypatch):
                 assert e.value.code == pw.PW_ECORRUPT
     model.close()
     codec.close()
+
+
+def _row(bank, tid):
+    """Table tid's packed index with centre 0 and its entries."""
+    t = tid // 128 - 8
+    return np.uint32(((t + (1 << 23)) << 7) | (tid % 128)), bank[tid]
+
+
+def test_lane_without_symbols_keeps_its_state(pw, codec, bank):
+    """One symbol on two lanes: the second lane's state has to be 2^16 as it
+    stands. A state of 1 that a spare zero word would lift to 2^16 is corrupt."""
+    pk, cdf = _row(bank, 8 * 128 + 20)
+    for r in (0, 1, -2, 7):
+        st, words = R.encode_chunk([R.symbol_ops(r, cdf)], 2)
+        idx = np.asarray([pk])
+        rc, got = _both(pw, codec, R.pack_chunk(st, words), 1, 2, idx)
+        assert rc == pw.PW_OK and got.tolist() == [r]
+        rc, _ = _both(pw, codec, R.pack_chunk([st[0], 1], words + [0]), 1, 2, idx)
+        assert rc == pw.PW_ECORRUPT
+
+
+@pytest.mark.parametrize("n", [1, 3, 8, 9, 30])
+def test_padded_rounds_read_no_words(pw, codec, bank, n):
+    """One lane whose state is 1 after its last symbol, and a spare zero word
+    (the rounds that fill up the last group of eight must not take it)."""
+    pk, cdf = _row(bank, 8 * 128 + 20)
+    s = R.T + 1                              # residual 0
+    c = int(cdf[s])
+    idx = np.full(n, pk)
+    # state c -> 0 -> the next word: c again (a symbol a word) or, last, 1
+    words = [c] * (n - 1)
+    rc, _ = _both(pw, codec, R.pack_chunk([c], words + [1, 0]), n, 1, idx)
+    assert rc == pw.PW_ECORRUPT
+    rc, _ = _both(pw, codec, R.pack_chunk([c], words + [1]), n, 1, idx)
+    assert rc == pw.PW_ECORRUPT
+    # the same symbols from a state that ends at 2^16 (c + 1 -> 1 -> 1 0000h):
+    # low states of lanes with symbols are the coder's business, and accepted
+    words = [c] * (n - 2) + [c + 1] if n > 1 else []
+    st = [c] if n > 1 else [c + 1]
+    out, used, xf = R.decode_chunk(st, words + [0], n, 1, lambda p: cdf)
+    assert out == [0] * n and used == n and xf == [R.L]
+    rc, got = _both(pw, codec, R.pack_chunk(st, words + [0]), n, 1, idx)
+    assert rc == pw.PW_OK and got.tolist() == [0] * n
