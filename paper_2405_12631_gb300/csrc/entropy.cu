@@ -194,7 +194,7 @@ constexpr uint32_t kResBytes = 2 * kRound * 32 * 4;      // residuals, 2 batches
 constexpr uint32_t kRing = 512, kFill = 384;     // words of the ring, of them loaded ahead
 constexpr uint32_t kRingBytes = 2 * (kRing + 32);   // (the first 32 words again at the end)
 constexpr uint32_t kPairBytes = kRowBufBytes + kResBytes + kRingBytes;
-constexpr int kMaxEscPasses = (2 * kMaxEscBits + 1) / 16 + 2;   // of up to 16 bypass bits
+constexpr int kMaxEscPasses = 2 * kMaxEscBits + 2;   // one bit each from states below 2^16
 constexpr uint32_t kRowGlobal = 0x80000000u;     // row entry: table id in global memory
 static_assert(2 * kNTables + 256 <= (int)kPairBytes, "row list and partial sums fit a pair area");
 
@@ -603,7 +603,7 @@ __global__ void __launch_bounds__(768) k_rans_decode(
                 if (!__any_sync(0xffffffffu, pend)) break;
                 bool nd = false;
                 if (pend) {
-                  const int n = max(1, 16 - __clz(x));   // x >= 2^16 in a valid stream
+                  const int n = max(1, 16 - __clz(x));
                   uint32_t bits = x >> 14;
                   int left = n;
                   if (!tail) {

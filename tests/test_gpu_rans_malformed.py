@@ -195,3 +195,27 @@ def test_padded_rounds_read_no_words(pw, codec, bank, n):
     assert out == [0] * n and used == n and xf == [R.L]
     rc, got = _both(pw, codec, R.pack_chunk(st, words + [0]), n, 1, idx)
     assert rc == pw.PW_OK and got.tolist() == [0] * n
+
+
+def test_low_states_between_escapes(pw, codec, bank):
+    """An escape read from states below 2^16, a word for every bit: the words
+    4000h give ones until a zero word ends the prefix."""
+    pk, cdf = _row(bank, 8 * 128 + 20)
+    c = int(cdf[R.ESC_R])
+    idx = np.asarray([pk])
+    for k in (1, 5, 6, 17, 30):
+        # c -> 0 -> 4000h (k times a one) -> 0 -> zero bit, then k bits of 0; the
+        # last word is 2^16's low half after 1 has been lifted: 4001h -> 1 on a one
+        words = [0x4000] * k + [0] + [0] * k
+        out, used, xf = R.decode_chunk([c], words + [0], 1, 1, lambda p: cdf)
+        e = (1 << k) - 1
+        assert out == [e + R.T + 1] and used == len(words) + 1
+        rc, got = _both(pw, codec, R.pack_chunk([c], words + [0]), 1, 1, idx)
+        # the end state is 0, not 2^16
+        assert xf == [0] and rc == pw.PW_ECORRUPT
+        words[-1] = 1
+        words.append(0)
+        out, used, xf = R.decode_chunk([c], words, 1, 1, lambda p: cdf)
+        assert out == [e + R.T + 1] and used == len(words) and xf == [R.L]
+        rc, got = _both(pw, codec, R.pack_chunk([c], words), 1, 1, idx)
+        assert rc == pw.PW_OK and got.tolist() == [e + R.T + 1]
