@@ -219,3 +219,21 @@ def test_low_states_between_escapes(pw, codec, bank):
         assert out == [e + R.T + 1] and used == len(words) and xf == [R.L]
         rc, got = _both(pw, codec, R.pack_chunk([c], words), 1, 1, idx)
         assert rc == pw.PW_OK and got.tolist() == [e + R.T + 1]
+
+
+@pytest.mark.parametrize("nl", [1, 8, 32])
+def test_corrupt_chunk_stops_early(pw, codec, bank, nl):
+    """Words that run out, or an escape that cannot be, end the chunk: what
+    lies far behind is not decoded (the output keeps its fill value)."""
+    rng = np.random.default_rng(nl)
+    n = 160 * nl
+    buf, idx, vals = _chunk(rng, bank, n, nl, {n // 2: 3})
+    rc, got = _both(pw, codec, buf, n, nl, idx)
+    assert rc == pw.PW_OK and got.tolist() == vals
+    cut = 4 * nl + 2 * ((len(buf) - 4 * nl) // 8)
+    rc, got = _both(pw, codec, buf[:cut], n, nl, idx)
+    assert rc == pw.PW_ECORRUPT and np.all(got[n * 3 // 4:] == -7)
+    buf, idx, vals = _chunk(rng, bank, n, nl, {n // 4: 40})
+    rc, got = _both(pw, codec, buf, n, nl, idx)
+    assert rc == pw.PW_ECORRUPT and np.all(got[n * 3 // 4:] == -7)
+    assert got[:n // 4 - 32 * nl].tolist() == vals[:n // 4 - 32 * nl]
