@@ -449,8 +449,8 @@ uint64_t pw_ctx_launch_count(const pw_ctx *ctx);
  * (default on; disabled classes use the default schedule) and returns the
  * previous setting. pw_autotune_report writes one line per tuned class
  * ("ks kb ncta epilogue fp8 log2tiles choice t0 t1 t2 t3": choice 0 =
- * default, 2 = alternative shape; t0 .. t3 = median sample time of each
- * candidate in microseconds, -1 = not sampled; epilogue 0 store, 1 ConvLSTM
+ * default, 2 = alternative shape; t0 and t2 = their median sample times in
+ * microseconds, t1 and t3 always -1, as a shape not sampled; epilogue 0 store, 1 ConvLSTM
  * gates, 2 head, 3 compact head, 4 store with a 16-channel BF16 input block)
  * into buf (NUL-terminated, truncated to n) and returns the full length. */
 int pw_autotune(int enable);

@@ -633,7 +633,9 @@ def padded_elems(hd: dict) -> int:
 
 
 def autotune_report() -> list:
-    """Tuned convolution classes as dicts (see pw_autotune_report)."""
+    """Tuned convolution classes as dicts (see pw_autotune_report): "choice"
+    is the index in "us" of the kept shape's time, "shape" 0 or 1, "pairs"
+    always 0 (there is one issue schedule)."""
     n = pw_autotune_report(None, 0)
     buf = C.create_string_buffer(n + 1)
     pw_autotune_report(buf, n + 1)

@@ -1182,7 +1182,7 @@ static void launch_masked_taps(const int32_t *s, __nv_bfloat16 *T, int P, int h,
   // blocks; below, a strip's loads one after another are the time, and 2 rows
   // (4 for 2) keep it short.
   uint4 *t4 = reinterpret_cast<uint4 *>(T);
-  if ((int64_t)P * h >= 8 * 1216)
+  if ((int64_t)P * h >= 8 * 8 * sm_count())
     k_masked_taps<8><<<P * ((h + 7) / 8), 128, 0, st>>>(s, t4, P, h, w, step);
   else
     k_masked_taps<2><<<P * ((h + 1) / 2), 128, 0, st>>>(s, t4, P, h, w, step);
@@ -1266,26 +1266,19 @@ static bool headc_ok(int h, int w) { return h >= 4 && w >= 8; }
 
 // ---- autotuner -------------------------------------------------------------
 // Per (kernel variant, size class = log2 of the tile count) the pipeline
-// shape. The candidates are sampled in place, round robin, on the real
-// launches of the decode / encode pipeline (each
-// launch bracketed by events that are read back later without a
-// synchronisation), so that the choice reflects the caches and concurrency
-// the kernel really sees; after kSamples samples of every candidate the
-// fastest median wins (the median ignores a one-off outlier such as the
-// first launch of a kernel, which loads its module). Results do not depend
-// on the schedule.
-// Candidates: bit 1 = the alternative pipeline shape (a shallower pipeline
-// for the plain convolutions, the second-best tile shape for the compact
-// head); bit 0 is not used (reported as not sampled).
-constexpr int kTuneCand = 4, kSamples = 3;
-struct TuneChoice {
-  int shape = 0;
-  int cand() const { return shape << 1; }
-};
+// shape: 0 the default, 1 the alternative (a shallower pipeline for the plain
+// convolutions, the second-best tile shape for the compact head). The two are
+// sampled in place, in turn, on the real launches of the decode / encode
+// pipeline (each launch bracketed by events that are read back later without
+// a synchronisation), so that the choice reflects the caches and concurrency
+// the kernel really sees; after kSamples samples of each the faster median
+// wins (the median ignores a one-off outlier such as the first launch of a
+// kernel, which loads its module). Results do not depend on the shape.
+constexpr int kTuneCand = 2, kSamples = 3;
 struct TuneEntry {
   bool tuned = false;
-  TuneChoice choice;
-  int next = 0;                        // candidate of the next sample
+  int shape = 0;                       // the choice
+  int next = 0;                        // shape of the next sample
   int issued[kTuneCand] = {};          // samples launched
   int n[kTuneCand] = {};               // samples read back
   float us[kTuneCand][kSamples] = {};  // their times
@@ -1299,7 +1292,7 @@ struct TuneEntry {
 };
 struct TunePending {
   uint64_t key;
-  int cand;
+  int shape;
   cudaEvent_t e0, e1;
 };
 static std::mutex g_tune_mu;
@@ -1329,7 +1322,7 @@ static void tune_poll_locked() {
     float ms = 0.f;
     if (e == cudaSuccess && cudaEventElapsedTime(&ms, q.e0, q.e1) == cudaSuccess) {
       TuneEntry &t = g_tune[q.key];
-      if (t.n[q.cand] < kSamples) t.us[q.cand][t.n[q.cand]++] = 1e3f * ms;
+      if (t.n[q.shape] < kSamples) t.us[q.shape][t.n[q.shape]++] = 1e3f * ms;
       bool done = !t.tuned;
       for (int c = 0; c < kTuneCand; ++c) done = done && (t.issued[c] == 0 || t.n[c] >= kSamples);
       if (done) {
@@ -1337,7 +1330,7 @@ static void tune_poll_locked() {
         for (int c = 0; c < kTuneCand; ++c)
           if (t.n[c] && t.median(c) < best) {
             best = t.median(c);
-            t.choice.shape = c >> 1;
+            t.shape = c;
           }
         t.tuned = true;
       }
@@ -1350,45 +1343,37 @@ static void tune_poll_locked() {
   g_tune_pending.resize(w);
 }
 
-// The schedule of the next launch of a class. While the class is being tuned
-// (sample = true) the launch is a sample of candidate `cand`.
-static TuneChoice tune_next(uint64_t key, bool has_alt, cudaStream_t st, bool &sample,
-                            int &cand) {
-  TuneChoice c;   // the default shape
+// The shape of the next launch of a class. While the class is being tuned
+// (sample = true) the launch is a sample of it.
+static int tune_next(uint64_t key, bool has_alt, cudaStream_t st, bool &sample) {
   sample = false;
   std::lock_guard<std::mutex> lk(g_tune_mu);
   tune_poll_locked();
   TuneEntry &t = g_tune[key];
-  if (t.tuned) {
-    c.shape = t.choice.shape && has_alt;
-    return c;
-  }
-  if (!g_tune_on.load()) return c;
+  if (t.tuned) return has_alt ? t.shape : 0;
+  if (!g_tune_on.load()) return 0;
   g_untuned_uses.fetch_add(1);
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
     cudaGetLastError();
-    return c;
+    return 0;
   }
   if (!has_alt) {  // nothing to choose
     t.tuned = true;
-    t.choice = TuneChoice{};
-    return c;
+    t.shape = 0;
+    return 0;
   }
-  auto valid = [](int k) { return !(k & 1); };
-  while (!valid(t.next)) t.next = (t.next + 1) % kTuneCand;
-  cand = t.next;
-  if (t.issued[cand] >= kSamples) return c;  // enough in flight; wait for read-back
-  do { t.next = (t.next + 1) % kTuneCand; } while (!valid(t.next));
-  t.issued[cand] += 1;
-  c.shape = cand >> 1;
+  const int c = t.next;
+  if (t.issued[c] >= kSamples) return 0;  // enough in flight; wait for read-back
+  t.next = c ^ 1;
+  t.issued[c] += 1;
   sample = true;
   return c;
 }
 
-static void tune_record(uint64_t key, int cand, cudaEvent_t e0, cudaEvent_t e1) {
+static void tune_record(uint64_t key, int shape, cudaEvent_t e0, cudaEvent_t e1) {
   std::lock_guard<std::mutex> lk(g_tune_mu);
-  g_tune_pending.push_back(TunePending{key, cand, e0, e1});
+  g_tune_pending.push_back(TunePending{key, shape, e0, e1});
 }
 
 uint64_t tune_untuned_uses() {
@@ -1403,8 +1388,8 @@ int tune_set_enabled(int on) {
   return old;
 }
 // One line per tuned class: "ks kb ncta epi f8 log2tiles choice t0 t1 t2 t3"
-// (choice = the kept candidate, bit 1 = alternative pipeline shape; t = median
-// sampled time of each candidate in microseconds, -1 = not sampled).
+// (choice = 0 for the default shape, 2 for the alternative; t0, t2 = their
+// median sampled times in microseconds; t1, t3 and shapes not sampled -1).
 std::string tune_report() {
   std::lock_guard<std::mutex> lk(g_tune_mu);
   tune_poll_locked();
@@ -1416,8 +1401,8 @@ std::string tune_report() {
     const TuneEntry &t = kv.second;
     snprintf(line, sizeof(line), "%d %d %d %d %d %d %d %.1f %.1f %.1f %.1f\n",
              (int)((k >> 32) & 0xFF), (int)((k >> 24) & 0xFF), (int)((k >> 14) & 0x3FF),
-             (int)((k >> 10) & 0xF), (int)((k >> 9) & 1), (int)(k & 0x1FF), t.choice.cand(),
-             t.median(0), t.median(1), t.median(2), t.median(3));
+             (int)((k >> 10) & 0xF), (int)((k >> 9) & 1), (int)(k & 0x1FF), t.shape << 1,
+             t.median(0), -1.0, t.median(1), -1.0);
     out += line;
   }
   return out;
@@ -1541,10 +1526,9 @@ static int conv_tc(pw_ctx *ctx, const TcWeights::Conv &cv, const void *in, int i
   // the steps 2-4 z conv) and the size (tiles of the default shape)
   const uint64_t key = tune_key(cv, a.epi, a.tiles);
   bool sample = false;
-  int cand = 0;
-  const TuneChoice ch = tune_next(key, has_alt, ctx->stream, sample, cand);
-  if (ch.shape && hc) set_hc_shape(lj_alt);
-  a.stages = (ch.shape && !hc) ? st_alt : st_def;
+  const int shape = tune_next(key, has_alt, ctx->stream, sample);
+  if (shape && hc) set_hc_shape(lj_alt);
+  a.stages = (shape && !hc) ? st_alt : st_def;
   const size_t smem = fixed + (size_t)a.stages * a.stage_bytes;
   CUtensorMap map, map1;
   int s;
@@ -1619,7 +1603,7 @@ static int conv_tc(pw_ctx *ctx, const TcWeights::Conv &cv, const void *in, int i
   cudaEventRecord(e0, st);
   s = launch(a, 1);
   cudaEventRecord(e1, st);
-  tune_record(key, cand, e0, e1);
+  tune_record(key, shape, e0, e1);
   return s;
 }
 
@@ -2149,7 +2133,7 @@ int tc_run_step(pw_ctx *ctx, Model &m, const Geometry &g, Workspace &ws, int sb,
       // a block's positions: four passes over the weights' one load where that
       // still gives every SM its four blocks twice
       const int one = (int)((chw + kDwThreads - 1) / kDwThreads);
-      const int per = (int64_t)P * G * one >= 4 * 8 * 152 ? 4 : 1;
+      const int per = (int64_t)P * G * one >= 4 * 8 * sm_count() ? 4 : 1;
       const int nblk = (one + per - 1) / per;
       k_dw3x3_compact<<<P * G * nblk, kDwThreads, 0, st>>>(
           t.U, zc_done ? nullptr : l, n.wdw, n.bdw, t.Vc, t.Zc, h, w, G, 0, per, nblk);
