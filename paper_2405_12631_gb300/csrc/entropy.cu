@@ -144,9 +144,9 @@ __device__ __forceinline__ void trio_sync(int id) {
 //
 // What bounds it: one dependent chain per chunk (state -> symbol -> state ->
 // shared word stream), a few hundred rounds long, one warp wide; the SMs are
-// otherwise idle. A round is laid out for the shortest chain (about 270
-// cycles, of them 60 the shared-memory load, 50 the shuffle and ballot, 25
-// the population count):
+// otherwise idle. A round is laid out for the shortest chain (it takes 0.16
+// us, about 330 cycles; of them about 35 are the shared-memory load, 45 the
+// shuffle and the ballot, 25 the population count):
 //  * The block first copies the table rows its symbols use (all indices of
 //    the pass are known) into shared memory, fine level and coarse level;
 //    rows beyond the shared memory's capacity, the ones whose scale is
@@ -1056,7 +1056,7 @@ void launch_rans_decode(const DecChunk *chunks, int nchunks, const uint16_t *ban
   });
   // chunks per block: one while every chunk finds an SM of its own, then as
   // many as that takes, up to 8 (24 warps; past that the shared-memory port is
-  // near its limit: 0.18 us a round for one chunk, 0.39 us for eight)
+  // near its limit: 0.16 us a round for one chunk, 0.31 us for eight)
   const int K = std::min(8, (nchunks + nsm - 1) / nsm);
   // table rows in shared memory: no more than the block has symbols (idx_stride
   // symbols a plane, 0 when unknown), so that small passes take little of it
