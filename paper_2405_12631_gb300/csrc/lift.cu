@@ -353,7 +353,8 @@ __device__ __forceinline__ bool lift_mma_wait(uint64_t *bar, uint32_t parity) {
 // (six resident CTAs per SM: 40 registers instead of 48, which allowed five;
 // lifting class 4.50 -> 4.45 ms per batch of 24. Layer 1 from the parameter
 // bank and on its 400 positions only: 4.36 -> 3.51 ms, with 4 bytes spilled;
-// what bounds it now is issue, 64 % of the slots.)
+// what bounds it now is issue (58 % of the slots with 2304 blocks) and the
+// waits between the phases of a tile.)
 __global__ void __launch_bounds__(256, 6) k_lift_tc(const __grid_constant__ LiftStepParams a,
                                                     const __grid_constant__ LiftTcWt wt) {
   extern __shared__ __align__(1024) uint8_t lsm_raw[];
