@@ -173,10 +173,10 @@ __device__ __forceinline__ void trio_sync(int id) {
 //    that was loaded one refill earlier.
 //  * Escapes and refills are looked for once per four rounds (a branch costs
 //    about 70 cycles of a round); see the loop.
-//  * A corrupt chunk (words run out, an escape beyond the limit) is decoded no
-//    further than the batch in which that branch finds it; after that its
-//    three warps only pass the barriers left. (Asked for at the head of every
-//    batch, it cost the cases 1.5 %.)
+//  * A corrupt chunk (words run out, an escape beyond the limit) ends where
+//    that branch finds it: the decoding warp passes the barriers left, and no
+//    further value is written. (Asked for at the head of every batch it cost
+//    the cases 1.5 %, by a variable loop bound 0.7 %; so, nothing.)
 // Measured, decoder launches alone, GB300: 3 chunks of 12,288 symbols on 32
 // lanes (384 rounds) 207 -> 68 us, of 4,096 (128 rounds) 72 -> 27 us, 192
 // chunks of 16,200 273 -> 98 us, 1,200 chunks of 16,384 453 -> 202 us, against
@@ -197,7 +197,7 @@ constexpr uint32_t kRowBufBytes = 3 * kRound * 32 * 4;   // row of each symbol, 
 constexpr uint32_t kResBytes = 2 * kRound * 32 * 4;      // residuals, 2 batches
 constexpr uint32_t kRing = 512, kFill = 384;     // words of the ring, of them loaded ahead
 constexpr uint32_t kRingBytes = 2 * (kRing + 32);   // (the first 32 words again at the end)
-constexpr uint32_t kStopOff = kRowBufBytes + kResBytes + kRingBytes;   // first batch not decoded
+constexpr uint32_t kStopOff = kRowBufBytes + kResBytes + kRingBytes;   // first batch not written
 constexpr uint32_t kPairBytes = kStopOff + 16;
 constexpr int kMaxEscPasses = 2 * kMaxEscBits + 2;   // one bit each from states below 2^16
 constexpr uint32_t kRowGlobal = 0x80000000u;     // row entry: table id in global memory
@@ -368,8 +368,8 @@ __global__ void __launch_bounds__(768) k_rans_decode(
   const int niter = (count + nl - 1) / nl;
   const int nbatch = (niter + kRound - 1) / kRound;
   const int bar = 1 + pr;
-  // first batch that is not decoded (batch b writes b + 1 or nothing, which the
-  // other warps see after barrier b + 1)
+  // first batch that is not written (batch b sets it to b or leaves it, which
+  // the third warp sees after barrier b + 1)
   volatile int *const stop = reinterpret_cast<volatile int *>(sm + pbase + kStopOff);
 
   if (role > 0) {
@@ -417,7 +417,7 @@ __global__ void __launch_bounds__(768) k_rans_decode(
       prepare(1);
       for (int b = 0; b < nbatch; ++b) {
         trio_sync(bar);
-        if (*stop > b) prepare(b + 2);
+        prepare(b + 2);
       }
       trio_sync(bar);
       return;
@@ -535,8 +535,7 @@ __global__ void __launch_bounds__(768) k_rans_decode(
     uint32_t row = 0, rown = 0;   // rows of the next round and the one after
     uint4 ca, cb;                 // coarse level of the next round
     uint32_t rb = rb0;            // row buffer of the batch
-    int b = 0, bend = nbatch;
-    for (; b < bend; ++b) {
+    for (int b = 0; b < nbatch; ++b) {
       trio_sync(bar);   // batches b and b + 1 prepared, the residuals of b - 2 consumed
       if (b == 0) {
         row = lds(rb);
@@ -662,15 +661,16 @@ __global__ void __launch_bounds__(768) k_rans_decode(
           }
           while (ptr + took - wb >= 64u) refill();
           if (__builtin_expect(__any_sync(0xffffffffu, bad || ptr + took > nwords), 0)) {
-            bend = b + 1;
-            if (lane == 0) *stop = bend;
+            if (lane == 0) *stop = b;
+            bad = true;
             __syncwarp();
+            for (; b < nbatch; ++b) trio_sync(bar);
+            return;
           }
         }
       }
       rb = rbn;
     }
-    for (; b < nbatch; ++b) trio_sync(bar);
     ptr += took;
     trio_sync(bar);
   };
