@@ -9,7 +9,7 @@
 // same layers in integer arithmetic, the head giving 16 mu and the scale
 // bin directly). The decoder runs one warp per plane
 // over the LL positions in raster order: the warp evaluates the model at the
-// next position from symbols already decoded, lane 0 decodes that symbol
+// next position from symbols already decoded, every lane decodes that symbol
 // from the plane's single-state rANS chunk and the warp moves on. The
 // encoder evaluates the same device function at every position in parallel
 // (all symbols known), so both sides derive bit-identical table indices.

@@ -1,6 +1,8 @@
-"""rANS decoder on hand-made chunks: escape prefixes up to the limit give
-their values, longer ones are reported. The oracle's coder writes the chunks
-from explicit coding operations, so that a prefix may have any length."""
+"""rANS decoder on hand-made chunks, as the oracle's coder writes them from
+explicit coding operations or as bare states and words: escape prefixes up to
+the limit give their values and longer ones are reported; lanes without a
+symbol read no words; states below 2^16 decode as the format defines; a
+corrupt chunk stops early."""
 import numpy as np
 import pytest
 
@@ -67,10 +69,10 @@ def _chunk(rng, bank, n, nl, escapes):
     return R.pack_chunk(st, words), idx, vals
 
 
-def _both(pw, codec, buf, n, nl, idx, nbytes=None):
+def _both(pw, codec, buf, n, nl, idx):
     """(status, values) of the regular and the allocation-free decoder."""
     u32 = lambda v: np.asarray([v], dtype=np.uint32)
-    a = (buf, u32(0), u32(len(buf) if nbytes is None else nbytes), u32(n), u32(nl), idx)
+    a = (buf, u32(0), u32(len(buf)), u32(n), u32(nl), idx)
     try:
         reg = pw.PW_OK, codec.rans_decode(*a)
     except pw.PwError as e:
